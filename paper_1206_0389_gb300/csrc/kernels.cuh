@@ -61,6 +61,9 @@ struct UpdateArgs {
   int pf_ahead;           // FP16 kernels: a CTA asks L2 for the block of work item
                           // it + pf_ahead (about half a wave ahead); 0 = off (set by
                           // the launcher)
+  int split;              // log2 of the runs a block's cells are cut into, each the work
+                          // of one CTA (set by the launcher)
+  int run_mask;           // cells (FP16 pairs) per run - 1 (set by the launcher)
 };
 
 // coarse-to-fine work comes in chunks of consecutive ghost cells (sorted by
