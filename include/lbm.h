@@ -13,7 +13,9 @@
  *   - Return value: LBM_OK (0) or a negative lbm_status.  Nothing throws.
  *     lbm_last_error() returns a message for the last failure on a context.
  *   - The context owns all device memory it allocates.  The caller owns every
- *     buffer it passes; host buffers may be pageable or pinned.
+ *     buffer it passes; host buffers may be pageable or pinned.  The dense
+ *     arrays of state, fields, force and gradients may also lie in memory of
+ *     the context's device; the caller's own work on them has to be done.
  *   - Calls are ordered on the context's stream.  lbm_step() only enqueues
  *     work; every call that returns data to the host synchronises the stream.
  *   - Dense per-level arrays are row-major with x fastest: index

@@ -239,8 +239,11 @@ struct SlabArgs {
   double* force;          // level body force [3][nblocks*512] or nullptr
   int ox, oy, oz, BX, BY, BZ;  // level box
   int NX, NY, z0, nz;
-  const double* in;       // SET_STATE: f [Q][n]; INIT_EQ: rho [n], u [3][n]; SET_FORCE: F [3][n]
-  double* out;            // GET_STATE: f [Q][n]; MACRO: rho [n], u [3][n]
+  // one dense array [nz][NY][NX] per component (n = NX NY nz values)
+  const double* in[27];   // SET_STATE: f_i; INIT_EQ: rho, u (nullptr: fill[c] everywhere);
+                          // SET_FORCE: F
+  double* out[27];        // GET_STATE: f_i; MACRO: rho, u
+  double fill[4];
   int mode;
   void* raw;              // SET_LAMBDA: [block][Q][512] (compute type); GET_FIELD3: [3][nblocks*512];
                           // GET_STATS: the statistics sums [7][nblocks*512] (double)
@@ -276,7 +279,9 @@ struct RadialArgs {
 };
 cudaError_t launch_radial(const RadialArgs& a, cudaStream_t st);
 cudaError_t launch_slab(int model, int storage, const SlabArgs& a, cudaStream_t st);
-cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t st);
+// ORs into *flags, shifted left by shift: 1 if any value is NaN, 2 if any is
+// infinite, 4 if any is not positive
+cudaError_t launch_check(const double* p, long long n, int shift, int* flags, cudaStream_t st);
 // float copy of a float64 array (the compute-type body force of FP32/FP16 storage)
 cudaError_t launch_to_float(const double* in, float* out, long long n, cudaStream_t st);
 
@@ -310,7 +315,6 @@ struct ReduceArgs {
   double* partial;   // [gridDim][4]
 };
 cudaError_t launch_reduce(int model, int storage, const ReduceArgs& a, int ctas, cudaStream_t st);
-cudaError_t launch_reduce_final(const double* partial, int n, double* out, int* nonfinite,
-                                cudaStream_t st);
+cudaError_t launch_reduce_final(const double* partial, int n, double* out, cudaStream_t st);
 
 }  // namespace lbm

@@ -38,7 +38,7 @@ __global__ void k_slab(const SlabArgs a) {
     case SLAB_SET_STATE: {
       if (j < 0) return;
       for (int i = 0; i < Q; ++i) {
-        const double v = a.in[int64_t(i) * n + t];
+        const double v = a.in[i][t];
         if (isnan(v)) continue;
         store_rt<S, Q>(f + i * kCells, i, T(v - shift_of<Q>(i)));
       }
@@ -46,13 +46,14 @@ __global__ void k_slab(const SlabArgs a) {
     }
     case SLAB_GET_STATE: {
       for (int i = 0; i < Q; ++i)
-        a.out[int64_t(i) * n + t] = j < 0 ? nan : double(load_rt<S, Q>(f + i * kCells, i)) + shift_of<Q>(i);
+        a.out[i][t] = j < 0 ? nan : double(load_rt<S, Q>(f + i * kCells, i)) + shift_of<Q>(i);
       return;
     }
     case SLAB_INIT_EQ: {
       if (j < 0) return;
-      const T rl = T(a.in[t] - 1.0);  // delta rho for both shifted models
-      const T ux = T(a.in[n + t]), uy = T(a.in[2 * n + t]), uz = T(a.in[3 * n + t]);
+      auto in = [&](int c) { return a.in[c] != nullptr ? a.in[c][t] : a.fill[c]; };
+      const T rl = T(in(0) - 1.0);  // delta rho for both shifted models
+      const T ux = T(in(1)), uy = T(in(2)), uz = T(in(3));
       T feq[Q];
       M::feq(rl, ux, uy, uz, feq);
       for (int i = 0; i < Q; ++i) store_rt<S, Q>(f + i * kCells, i, feq[i]);
@@ -61,7 +62,7 @@ __global__ void k_slab(const SlabArgs a) {
     case SLAB_MACRO: {
       const uint8_t k = j < 0 ? uint8_t(K_NONE) : a.kind[j];
       if (k != K_ACTIVE && k != K_HIDDEN1 && k != K_HIDDEN2) {
-        for (int c = 0; c < 4; ++c) a.out[c * n + t] = nan;
+        for (int c = 0; c < 4; ++c) a.out[c][t] = nan;
         return;
       }
       double g[Q];
@@ -86,22 +87,22 @@ __global__ void k_slab(const SlabArgs a) {
         uy = jy / rho;
         uz = jz / rho;
       }
-      a.out[t] = rho;
-      a.out[n + t] = ux;
-      a.out[2 * n + t] = uy;
-      a.out[3 * n + t] = uz;
+      a.out[0][t] = rho;
+      a.out[1][t] = ux;
+      a.out[2][t] = uy;
+      a.out[3][t] = uz;
       return;
     }
     case SLAB_SET_LAMBDA: {
       if (j < 0) return;
       T* r = reinterpret_cast<T*>(a.raw) + blk * Q * kCells + cell;
-      for (int i = 0; i < Q; ++i) r[i * kCells] = T(a.in[int64_t(i) * n + t]);
+      for (int i = 0; i < Q; ++i) r[i * kCells] = T(a.in[i][t]);
       return;
     }
     case SLAB_GET_FIELD3: {
       const int64_t nn = int64_t(a.BX) * a.BY * a.BZ * kCells;
       const T* r = reinterpret_cast<const T*>(a.raw);
-      for (int c = 0; c < 3; ++c) a.out[c * n + t] = j < 0 ? nan : double(r[c * nn + j]);
+      for (int c = 0; c < 3; ++c) a.out[c][t] = j < 0 ? nan : double(r[c * nn + j]);
       return;
     }
     case SLAB_GET_STATS: {
@@ -110,26 +111,26 @@ __global__ void k_slab(const SlabArgs a) {
       const bool ok = k == K_ACTIVE || k == K_HIDDEN1 || k == K_HIDDEN2;
       const int64_t nn = int64_t(a.BX) * a.BY * a.BZ * kCells;
       const double* r = reinterpret_cast<const double*>(a.raw);
-      for (int c = 0; c < 4; ++c) a.out[c * n + t] = ok ? r[c * nn + j] * a.scale : nan;
+      for (int c = 0; c < 4; ++c) a.out[c][t] = ok ? r[c * nn + j] * a.scale : nan;
       for (int c = 0; c < 3; ++c) {
         const double m = ok ? r[(1 + c) * nn + j] * a.scale : 0.0;
-        a.out[(4 + c) * n + t] = ok ? r[(4 + c) * nn + j] * a.scale - m * m : nan;
+        a.out[4 + c][t] = ok ? r[(4 + c) * nn + j] * a.scale - m * m : nan;
       }
       return;
     }
     case SLAB_GET_AUX: {
-      a.out[t] = j < 0 ? nan : double(reinterpret_cast<const T*>(a.raw)[j]);
+      a.out[0][t] = j < 0 ? nan : double(reinterpret_cast<const T*>(a.raw)[j]);
       return;
     }
     case SLAB_SET_AUX: {
-      if (j < 0 || isnan(a.in[t])) return;
-      reinterpret_cast<T*>(a.raw)[j] = T(a.in[t]);
+      if (j < 0 || isnan(a.in[0][t])) return;
+      reinterpret_cast<T*>(a.raw)[j] = T(a.in[0][t]);
       return;
     }
     case SLAB_SET_FORCE: {
       if (j < 0) return;
       const int64_t nn = int64_t(a.BX) * a.BY * a.BZ * kCells;
-      for (int c = 0; c < 3; ++c) a.force[c * nn + j] = a.in[c * n + t];
+      for (int c = 0; c < 3; ++c) a.force[c * nn + j] = a.in[c][t];
       return;
     }
   }
@@ -278,13 +279,13 @@ __global__ void __launch_bounds__(256, reduce_ctas_per_sm(std::is_same<S, __half
   }
 }
 
-__global__ void k_reduce_final(const double* partial, int n, double* out, int* nonfinite) {
-  if (threadIdx.x < 4) {
-    double v = 0;
-    for (int i = 0; i < n; ++i) v += partial[i * 4 + threadIdx.x];
-    out[threadIdx.x] = v;
-    if (!isfinite(v)) atomicExch(nonfinite, 1);
-  }
+// one warp per sum; out may be registered host memory
+__global__ void k_reduce_final(const double* partial, int n, double* out) {
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0;
+  for (int i = lane; i < n; i += 32) v += partial[i * 4 + c];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (lane == 0) out[c] = v;
 }
 
 template <class M, class S>
@@ -321,9 +322,20 @@ cudaError_t launch_gather(int model, int storage, const GatherArgs& a, cudaStrea
 cudaError_t launch_reduce(int model, int storage, const ReduceArgs& a, int ctas, cudaStream_t st) {
   LBM_DISPATCH(reduce_ms, a, ctas, st)
 }
-__global__ void k_fill(double* p, long long n, double v) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) p[t] = v;
+// input checks: four loads in flight per thread (the values may lie in host
+// memory, a link away)
+__global__ void __launch_bounds__(256) k_check(const double* p, long long n, int shift, int* flags) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  int f = 0;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += 4 * stride) {
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = t + k * stride < n ? p[t + k * stride] : 1.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f |= (isnan(v[k]) ? 1 : 0) | (isinf(v[k]) ? 2 : 0) | (v[k] > 0 ? 0 : 4);
+  }
+  f = __reduce_or_sync(0xffffffffu, unsigned(f));
+  if (f && (threadIdx.x & 31) == 0) atomicOr(flags, f << shift);
 }
 // one sample of the time statistics: rho and u of every cell holding a value
 // of the level (the same moments as the macroscopic output), accumulated in
@@ -418,14 +430,15 @@ cudaError_t launch_to_float(const double* in, float* out, long long n, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_fill<<<unsigned((n + 255) / 256), 256, 0, st>>>(p, n, v);
+cudaError_t launch_check(const double* p, long long n, int shift, int* flags, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  const long long ctas = (n + 1023) / 1024;
+  k_check<<<unsigned(ctas < 4096 ? ctas : 4096), 256, 0, st>>>(p, n, shift, flags);
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_final(const double* partial, int n, double* out, int* nonfinite, cudaStream_t st) {
-  k_reduce_final<<<1, 32, 0, st>>>(partial, n, out, nonfinite);
+cudaError_t launch_reduce_final(const double* partial, int n, double* out, cudaStream_t st) {
+  k_reduce_final<<<1, 128, 0, st>>>(partial, n, out);
   return cudaGetLastError();
 }
 
