@@ -34,7 +34,7 @@ namespace {
 thread_local std::string g_create_error;
 
 struct Op {
-  enum Kind { UPDATE, C2F, F2C, BC, LINK, INC } kind;
+  enum Kind { UPDATE, C2F, F2C, BC, LINK } kind;
   int k = 0;            // finest-level substep of the coarse step the op belongs to
   bool level0 = false;  // an update of level-0 blocks alone (first substep of a nested grid)
   UpdateArgs ua{};
@@ -96,8 +96,8 @@ struct lbm_ctx {
   uint64_t seed = 0;
   // launch configuration
   int threads = 256, minb = 1, ctas = 0;
-  // graphs, one per level-0 parity
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  // graphs of one and of kManySteps coarse steps, one per level-0 parity
+  cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
   bool graphs_valid = false;
   bool profiling = false;
   // adjoint: checkpoints every `every` steps, segment buffers, lambda, dL/dF
@@ -161,9 +161,15 @@ void release_adjoint(lbm_ctx* c) {
   c->adj_ready = false;
 }
 
+void drop_graphs(lbm_ctx* c) {
+  for (cudaGraphExec_t* g : {&c->graph[0], &c->graph[1], &c->many[0], &c->many[1]}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+}
+
 void free_all(lbm_ctx* c) {
-  for (int p = 0; p < 2; ++p)
-    if (c->graph[p]) cudaGraphExecDestroy(c->graph[p]);
+  drop_graphs(c);
   for (DevLevel& d : c->dl) {
     cudaFree(d.f[0]);
     cudaFree(d.f[1]);
@@ -344,6 +350,13 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
                                        : static_cast<const void*>(c->dl[0].force_f);
     u.walls = c->plan.walls;
     u.slip = c->plan.slip;
+    // only the inflow reads the step counter, before the last update
+    u.step_inc = k == K - 1 && !c->plan.periodic_x ? c->d_step : nullptr;
+    // a coarse step of one level without ghosts is this launch alone.  FP64
+    // storage, bound by the float64 pipes, waits for the launch to end: CTAs
+    // that come in among the last of the step before spread unevenly over the
+    // SMs (32^3 D3Q19: 16.8 us per step, chained 22.7)
+    u.chained = L == 1 && c->plan.periodic_x && c->storage != LBM_F64;
     up.k = k;
     if (lmin == 0 && split_level0(c)) {
       // the first substep updates level 0 in a launch of its own: nothing
@@ -390,10 +403,6 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
       if (a.n > 0) ops.push_back(op);
     }
   }
-  Op inc;
-  inc.k = K - 1;
-  inc.kind = Op::INC;
-  ops.push_back(inc);
   return ops;
 }
 
@@ -404,7 +413,6 @@ cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st) {
     case Op::F2C: return launch_f2c(c->model, c->storage, op.fa, st);
     case Op::BC: return launch_bc(c->model, c->storage, op.ba, st);
     case Op::LINK: return launch_links(c->model, c->storage, op.la, st);
-    case Op::INC: return launch_step_inc(c->d_step, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -417,8 +425,8 @@ int op_kind_index(const Op& op) {
     case Op::F2C: return 2;
     case Op::BC:
     case Op::LINK: return 3;
-    default: return 4;
   }
+  return 4;
 }
 
 // restriction of every hidden layer from the current fine state (after an
@@ -445,17 +453,20 @@ int restrict_all(lbm_ctx* ctx) {
   return LBM_OK;
 }
 
-int build_graphs(lbm_ctx* ctx) {
+// Short coarse steps (small grids) are bound by the launch of a graph per
+// step, so a run of steps goes out as graphs of kManySteps steps: 53,760 cells
+// of D3Q27 FP32 8.4 -> 4.4 us per step, 96^3 36.9 -> 31.3, 256^3 FP16 309 -> 300
+// (with the chained launches of begin_update).  The number is even: the parity comes round.
+constexpr int kManySteps = 16;
+
+// captures `steps` coarse steps that start at level-0 parity p0
+int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
   const int K = 1 << (ctx->L - 1);
-  for (int p = 0; p < 2; ++p) {
-    if (ctx->graph[p]) {
-      cudaGraphExecDestroy(ctx->graph[p]);
-      ctx->graph[p] = nullptr;
-    }
-    std::vector<Op> ops = build_schedule(ctx, p);
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
+  cudaGraph_t g = nullptr;
+  CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = cudaSuccess;
+  for (int s = 0; s < steps && e == cudaSuccess; ++s) {
+    std::vector<Op> ops = build_schedule(ctx, p0 ^ (s & 1));
     size_t ev = 0;
     auto next_event = [&](cudaEvent_t* out) {
       if (ev >= ctx->fork_join.size()) return cudaErrorInvalidValue;
@@ -530,20 +541,32 @@ int build_graphs(lbm_ctx* ctx) {
       if (e == cudaSuccess && (e = next_event(&evt)) == cudaSuccess && (e = cudaEventRecord(evt, st)) == cudaSuccess)
         e = cudaStreamWaitEvent(ctx->stream, evt, 0);
     }
-    cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
-    if (e != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      return cuda_fail(ctx, e, "capture");
-    }
-    if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
-    // kernel nodes carry the priority of the stream they were captured from
-    e = cudaGraphInstantiateWithFlags(&ctx->graph[p], g, cudaGraphInstantiateFlagUseNodePriority);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiateWithFlags");
   }
+  cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return cuda_fail(ctx, e, "capture");
+  }
+  if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
+  // kernel nodes carry the priority of the stream they were captured from
+  e = cudaGraphInstantiateWithFlags(exec, g, cudaGraphInstantiateFlagUseNodePriority);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    *exec = nullptr;
+    return cuda_fail(ctx, e, "cudaGraphInstantiateWithFlags");
+  }
+  return LBM_OK;
+}
+
+// the graphs of single steps; those of kManySteps are captured when first used
+int build_graphs(lbm_ctx* ctx) {
+  drop_graphs(ctx);
+  for (int p = 0; p < 2; ++p)
+    if (int rc = capture_steps(ctx, p, 1, &ctx->graph[p])) return rc;
   ctx->graphs_valid = true;
   return LBM_OK;
 }
+
 
 // Pick the stream-collide launch shape by timing the largest update launch of
 // the schedule: threads per CTA in {128, 256} with register caps, one CTA per block or a
@@ -556,6 +579,8 @@ int autotune(lbm_ctx* ctx) {
   for (const Op& op : ops)
     if (op.kind == Op::UPDATE && (!big || op.ua.nitems > big->ua.nitems)) big = &op;
   if (!big || big->ua.nitems == 0) return LBM_OK;
+  UpdateArgs trial = big->ua;
+  trial.step_inc = nullptr;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -587,18 +612,23 @@ int autotune(lbm_ctx* ctx) {
     if (update_occupancy(ctx->model, ctx->storage, ctx->plan.walls != 0, t, mb, &occ) != cudaSuccess || occ < 1) continue;
     const int clist[2] = {0, occ * ctx->sms};
     for (int cc : clist) {
-      if (launch_update(ctx->model, ctx->storage, big->ua, t, mb, cc, ctx->stream) != cudaSuccess) continue;
-      CK(launch_update(ctx->model, ctx->storage, big->ua, t, mb, cc, ctx->stream));
-      // best of three groups of four launches
+      // a list that is resident as a whole makes the same launch either way
+      if (cc > 0 && trial.nitems <= (ctx->storage == LBM_F64 ? cc / 4 : cc)) continue;
+      if (launch_update(ctx->model, ctx->storage, trial, t, mb, cc, ctx->stream) != cudaSuccess) continue;
+      CK(launch_update(ctx->model, ctx->storage, trial, t, mb, cc, ctx->stream));
+      // best of three groups of launches, each of 4 or as many as take 60 us
+      // (the shapes of a small grid differ by less than the jitter of four)
       float ms = 1e30f;
-      for (int grp = 0; grp < 3; ++grp) {
+      int reps = 4;
+      for (int grp = 0; grp < 4; ++grp) {
         CK(cudaEventRecord(e0, ctx->stream));
-        for (int r = 0; r < 4; ++r) CK(launch_update(ctx->model, ctx->storage, big->ua, t, mb, cc, ctx->stream));
+        for (int r = 0; r < reps; ++r) CK(launch_update(ctx->model, ctx->storage, trial, t, mb, cc, ctx->stream));
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaEventSynchronize(e1));
         float g = 0;
         CK(cudaEventElapsedTime(&g, e0, e1));
-        ms = std::min(ms, g);
+        if (grp > 0) ms = std::min(ms, g / float(reps));
+        else reps = std::max(4, std::min(64, int(0.06f * float(reps) / std::max(g, 1e-3f))));
       }
       if (ms < best) {
         best = ms;
@@ -1107,7 +1137,16 @@ int lbm_step(lbm_ctx* ctx, int coarse_steps) {
     int rc = build_graphs(ctx);
     if (rc) return rc;
   }
-  for (int n = 0; n < coarse_steps; ++n) {
+  int left = coarse_steps;
+  if (left >= kManySteps && !ctx->many[ctx->parity0]) {
+    int rc = capture_steps(ctx, ctx->parity0, kManySteps, &ctx->many[ctx->parity0]);
+    if (rc) return rc;
+  }
+  for (; left >= kManySteps; left -= kManySteps) {
+    CK(cudaGraphLaunch(ctx->many[ctx->parity0], ctx->stream));
+    ctx->step += kManySteps;
+  }
+  for (; left > 0; --left) {
     CK(cudaGraphLaunch(ctx->graph[ctx->parity0], ctx->stream));
     ctx->parity0 ^= 1;
     ctx->step++;

@@ -451,8 +451,6 @@ __global__ void __launch_bounds__(128) k_links(const LinkArgs a) {
   store_rt<S, Q>(f + int64_t(it.bblock) * QS + ib * kCells + it.bcell, ib, v);
 }
 
-__global__ void k_step_inc(long long* step) { *step += 1; }
-
 // coarse-to-fine: one CTA per chunk; fine-to-coarse: four lanes per item, 32
 // items per CTA; inflow: eight lanes per item, 16 items per CTA
 template <class M, class S>
@@ -494,10 +492,5 @@ cudaError_t launch_c2f(int model, int storage, const C2FArgs& a, cudaStream_t st
 cudaError_t launch_f2c(int model, int storage, const F2CArgs& a, cudaStream_t st) { LBM_DISPATCH(f2c_ms, a, st) }
 cudaError_t launch_bc(int model, int storage, const BCArgs& a, cudaStream_t st) { LBM_DISPATCH(bc_ms, a, st) }
 cudaError_t launch_links(int model, int storage, const LinkArgs& a, cudaStream_t st) { LBM_DISPATCH(links_ms, a, st) }
-
-cudaError_t launch_step_inc(long long* step, cudaStream_t st) {
-  k_step_inc<<<1, 1, 0, st>>>(step);
-  return cudaGetLastError();
-}
 
 }  // namespace lbm

@@ -63,6 +63,10 @@ struct UpdateArgs {
                           // the launcher)
   int split;              // log2 of the runs a block's cells are cut into, each the work
                           // of one CTA (set by the launcher)
+  long long* step_inc;    // coarse-step counter that the last update of a coarse step
+                          // advances (nothing after it in the step reads it), or nullptr
+  int chained;            // the launch may begin while the launch before it, an update
+                          // too, still ends (programmatic dependent launch)
   int run_mask;           // cells (FP16 pairs) per run - 1 (set by the launcher)
 };
 
@@ -227,7 +231,6 @@ cudaError_t launch_c2f(int model, int storage, const C2FArgs& a, cudaStream_t st
 cudaError_t launch_f2c(int model, int storage, const F2CArgs& a, cudaStream_t st);
 cudaError_t launch_bc(int model, int storage, const BCArgs& a, cudaStream_t st);
 cudaError_t launch_links(int model, int storage, const LinkArgs& a, cudaStream_t st);
-cudaError_t launch_step_inc(long long* step, cudaStream_t st);
 
 // dense <-> block staging for one slab of cell layers [z0, z0 + nz) of a level
 enum SlabMode { SLAB_SET_STATE = 0, SLAB_GET_STATE = 1, SLAB_INIT_EQ = 2, SLAB_MACRO = 3,
