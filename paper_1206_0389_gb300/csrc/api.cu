@@ -340,6 +340,7 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
       u.lv[l].BY = lp.BY;
       u.lv[l].BZ = lp.BZ;
       u.lv[l].tau0 = lp.tau0;
+      u.lv[l].omega = c->storage == LBM_F64 ? 1.0 / lp.tau0 : double(1.0f / float(lp.tau0));
     }
     u.items = c->items + c->list_off[lmin];
     u.nitems = int(c->list_len[lmin]);

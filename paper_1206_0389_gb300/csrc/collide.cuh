@@ -8,6 +8,8 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "lattice.cuh"
 
 namespace lbm {
@@ -231,40 +233,6 @@ __device__ __forceinline__ void inv_line(T& a, T& b, T& c, T u, T uu, T K) {
 }
 
 template <class T>
-__device__ __forceinline__ void forward27(T (&v)[3][3][3], T ux, T uy, T uz) {
-  const T ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) fwd_line(v[i][j][0], v[i][j][1], v[i][j][2], uz, uz2, T(w1(i) * w1(j)));
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) fwd_line(v[i][0][k], v[i][1][k], v[i][2][k], uy, uy2, T(w1(i) * c1(k)));
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) fwd_line(v[0][j][k], v[1][j][k], v[2][j][k], ux, ux2, T(c1(j) * c1(k)));
-}
-
-template <class T>
-__device__ __forceinline__ void inverse27(T (&v)[3][3][3], T ux, T uy, T uz) {
-  const T ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) inv_line(v[0][j][k], v[1][j][k], v[2][j][k], ux, ux2, T(c1(j) * c1(k)));
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) inv_line(v[i][0][k], v[i][1][k], v[i][2][k], uy, uy2, T(w1(i) * c1(k)));
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) inv_line(v[i][j][0], v[i][j][1], v[i][j][2], uz, uz2, T(w1(i) * w1(j)));
-}
-
-template <class T>
 __device__ __forceinline__ void to_cube(const T* g, T (&v)[3][3][3]) {
   static_for<27>([&](auto i) { v[D3Q27::ex(i) + 1][D3Q27::ey(i) + 1][D3Q27::ez(i) + 1] = g[i]; });
 }
@@ -290,56 +258,8 @@ __device__ __forceinline__ void moments27(const T* g, T& drho, T& jx, T& jy, T& 
 // from the post-collision second-order moments (third and fifth order 0,
 // fourth M_aa M_bb and M_aa M_bc, sixth M11 M22 M33).  With a body force F,
 // u = (j + F/2)/rho and the first central moments leave as F/(2 rho).
-template <class T>
-__device__ __forceinline__ void collide27(T* g, T omega, T Fx, T Fy, T Fz) {
-  T drho, jx, jy, jz;
-  moments27(g, drho, jx, jy, jz);
-  const T rho = T(1) + drho;
-  const T irho = T(1) / rho;
-  const T ux = (jx + T(0.5) * Fx) * irho, uy = (jy + T(0.5) * Fy) * irho, uz = (jz + T(0.5) * Fz) * irho;
-  T v[3][3][3];
-  to_cube(g, v);
-  forward27(v, ux, uy, uz);
-  const T om1 = T(1) - omega;
-  const T mean = (v[2][0][0] + v[0][2][0] + v[0][0][2]) * T(1.0 / 3.0);
-  const T Dx = om1 * (v[2][0][0] - mean) * irho;
-  const T Dy = om1 * (v[0][2][0] - mean) * irho;
-  const T Dz = om1 * (v[0][0][2] - mean) * irho;
-  const T kxy = om1 * v[1][1][0], kxz = om1 * v[1][0][1], kyz = om1 * v[0][1][1];  // rho kappa'
-  const T third = T(1.0 / 3.0);
-  const T Xx = third + Dx, Yy = third + Dy, Zz = third + Dz;  // kappa'_200 ...
-  // zeroth and first order
-  v[0][0][0] = drho;
-  v[1][0][0] = T(0.5) * Fx;
-  v[0][1][0] = T(0.5) * Fy;
-  v[0][0][1] = T(0.5) * Fz;
-  // second order
-  v[2][0][0] = drho * third + rho * Dx;
-  v[0][2][0] = drho * third + rho * Dy;
-  v[0][0][2] = drho * third + rho * Dz;
-  v[1][1][0] = kxy;
-  v[1][0][1] = kxz;
-  v[0][1][1] = kyz;
-  // third order
-  v[2][1][0] = v[2][0][1] = v[1][2][0] = v[0][2][1] = v[1][0][2] = v[0][1][2] = v[1][1][1] = T(0);
-  // fourth order
-  const T ninth = T(1.0 / 9.0);
-  v[2][2][0] = drho * ninth + rho * ((Dx + Dy) * third + Dx * Dy);
-  v[2][0][2] = drho * ninth + rho * ((Dx + Dz) * third + Dx * Dz);
-  v[0][2][2] = drho * ninth + rho * ((Dy + Dz) * third + Dy * Dz);
-  v[2][1][1] = Xx * kyz;
-  v[1][2][1] = Yy * kxz;
-  v[1][1][2] = Zz * kxy;
-  // fifth order
-  v[2][2][1] = v[2][1][2] = v[1][2][2] = T(0);
-  // sixth order
-  v[2][2][2] = drho * T(1.0 / 27.0) +
-               rho * ((Dx + Dy + Dz) * ninth + (Dx * Dy + Dx * Dz + Dy * Dz) * third + Dx * Dy * Dz);
-  inverse27(v, ux, uy, uz);
-  from_cube(v, g);
-}
-
-// The same collision in closed form, used by the stream-collide kernel.
+//
+// In closed form, used by the stream-collide kernel with FP32 storage.
 // Because every moment above second order is relaxed with rate 1, only the
 // six pre-collision second-order central moments matter; they follow from
 // raw sums: rho kappa_aa = S_aa - 2 u_a j_a + u_a^2 rho (+ const), rho kappa_ab =
@@ -353,10 +273,7 @@ __device__ __forceinline__ void collide27(T* g, T omega, T Fx, T Fy, T Fz) {
 // keeps f* - w free of cancellation:
 //   f*_i - w_i = drho W_i + rho (dx Py Pz... expanded) + k_xy psi_x psi_y phi_z + ...
 // (the paper notes that fixed rates remove most of the FCLB flops).
-// Scaled: g holds g_i / w_i on entry and exit (the FP16 storage form); the
-// product weights w_i = w1_x w1_y w1_z then enter once per z-line on input
-// and once per (e_y, e_z) pair and per e_x factor on output.
-template <class T, bool Force, bool Scaled = false>
+template <class T, bool Force>
 __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz) {
   // ---- zeroth, first and second raw moments of g by a z, y, x collapse
   T m0[3][3], dz[3][3], sz[3][3];  // per (ex, ey): sum, difference, sum of ends along z
@@ -367,16 +284,9 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
       const T lo = g[D3Q27::index(a - 1, b - 1, -1)];
       const T mi = g[D3Q27::index(a - 1, b - 1, 0)];
       const T hi = g[D3Q27::index(a - 1, b - 1, 1)];
-      if constexpr (Scaled) {
-        const T ce = T(w1(a) * w1(b) * w1(0)), cm = T(w1(a) * w1(b) * w1(1));
-        sz[a][b] = ce * (hi + lo);
-        dz[a][b] = ce * (hi - lo);
-        m0[a][b] = sz[a][b] + cm * mi;
-      } else {
-        sz[a][b] = hi + lo;
-        dz[a][b] = hi - lo;
-        m0[a][b] = sz[a][b] + mi;
-      }
+      sz[a][b] = hi + lo;
+      dz[a][b] = hi - lo;
+      m0[a][b] = sz[a][b] + mi;
     }
   T M0[3], My[3], Myy[3], Dz[3], Dyz[3], Szz[3];
 #pragma unroll
@@ -444,47 +354,20 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
     }
   }
   // ---- per (e_y, e_z) pair, then per e_x
-  if constexpr (Scaled) {
-    // the x factors divided by w1_x once
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      dl[0][a] *= T(1.0 / w1(a));
-      ps[0][a] *= T(1.0 / w1(a));
-      ph[0][a] *= T(1.0 / w1(a));
-      if constexpr (Force) ch[0][a] *= T(1.0 / w1(a));
-    }
-  }
 #pragma unroll
   for (int b = 0; b < 3; ++b)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const T P = ph[1][b] * ph[2][c];                            // phi_y phi_z
       const T Qd = T(w1(b)) * dl[2][c] + dl[1][b] * ph[2][c];     // phi_y phi_z - w1_y w1_z
-      T rP = rho * P, rQ = rho * Qd;
-      T R = kxy * ps[1][b] * ph[2][c] + kxz * ph[1][b] * ps[2][c];
-      T Sy = kyz * ps[1][b] * ps[2][c];
+      const T rP = rho * P, rQ = rho * Qd;
+      const T R = kxy * ps[1][b] * ph[2][c] + kxz * ph[1][b] * ps[2][c];
+      const T Sy = kyz * ps[1][b] * ps[2][c];
       T Fp = T(0), Gp = T(0);
       if constexpr (Force) {
         Fp = T(0.5) * Fx * ch[1][b] * ch[2][c];
         Gp = T(0.5) * Fy * ps[1][b] * ch[2][c] + T(0.5) * Fz * ch[1][b] * ps[2][c];
       }
-      if constexpr (Scaled) {
-        const T ibc = T(1.0 / (w1(b) * w1(c)));
-        rP *= ibc;
-        R *= ibc;
-        Sy *= ibc;
-        if constexpr (Force) {
-          Fp *= ibc;
-          Gp *= ibc;
-        }
-        const T base = drho + ibc * rQ;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          T v = base + dl[0][a] * rP + ps[0][a] * R + ph[0][a] * Sy;
-          if constexpr (Force) v += ps[0][a] * Fp + ch[0][a] * Gp;
-          g[D3Q27::index(a - 1, b - 1, c - 1)] = v;
-        }
-      } else {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           const T W = T(w1(a) * w1(b) * w1(c));
@@ -492,8 +375,174 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
           if constexpr (Force) v += ps[0][a] * Fp + ch[0][a] * Gp;
           g[D3Q27::index(a - 1, b - 1, c - 1)] = v;
         }
-      }
     }
+}
+
+// The collision of collide27_closed as nested one-dimensional lines, for FP64
+// and FP16 storage.  A line is the three values along one axis of
+//   c w1(e) + A delta(e) + R psi(e),   delta(+-1) = E +- u/2, delta(0) = -2 E,
+//   psi(+-1) = u +- 1/2, psi(0) = -2 u,  E = (u^2 + D) / 2,
+// which come in pairs: with t = E A + u R the even part is c/6 + t, the odd
+// part u A + R, and the centre c - 2 (c/6 + t), so a line takes 7 operations
+// and its sum is c by construction.  Along z the slots are (drho, rho, 0); each
+// value c found gives the next axis its A = c + w, and kyz psi_z its R; the
+// shear terms kxy phi_z, kxz psi_z make a second line along y that is the R of
+// the x lines.  About 245 operations a cell against 400 of collide27_closed,
+// and fewer values alive (112 registers against 212 in float64 without a cap):
+// 128^3 FP64, bound by the float64 pipes, 1313 -> 1006 us per step; 256^3 FP16
+// 300 -> 287 us.  The last bits differ, so FP32 storage, bound by memory,
+// keeps that form.
+// Scaled (FP16 storage): values are g_i / w_i; all sums run in units of
+// products of 1/6 (a middle value weighs 4, exactly) and lines have no weights.
+// om1 = 1 - omega.
+template <class T, bool Scaled>
+__device__ __forceinline__ void emit_line(T c, T t, T odd, T& lo, T& mid, T& hi) {
+  if constexpr (Scaled) {
+    mid = c - T(3) * t;
+    const T ev = c + T(6) * t;
+    lo = ev - T(3) * odd;
+    hi = ev + T(3) * odd;
+  } else {
+    const T ev = T(1.0 / 6.0) * c + t;
+    mid = c - T(2) * ev;
+    lo = ev - T(0.5) * odd;
+    hi = ev + T(0.5) * odd;
+  }
+}
+template <class T, bool Force, bool Scaled>
+__device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
+  // ---- raw moments up to second order by a z, y, x collapse
+  auto centre = [](T ends, T mid) -> T {
+    if constexpr (Scaled) return T(4) * mid + ends;
+    else return ends + mid;
+  };
+  T m0[3][3], dz[3][3], sz[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const T lo = g[D3Q27::index(a - 1, b - 1, -1)], hi = g[D3Q27::index(a - 1, b - 1, 1)];
+      sz[a][b] = hi + lo;
+      dz[a][b] = hi - lo;
+      m0[a][b] = centre(sz[a][b], g[D3Q27::index(a - 1, b - 1, 0)]);
+    }
+  T M0[3], My[3], Myy[3], Dz[3], Dyz[3], Szz[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    Myy[a] = m0[a][2] + m0[a][0];
+    My[a] = m0[a][2] - m0[a][0];
+    M0[a] = centre(Myy[a], m0[a][1]);
+    Dz[a] = centre(dz[a][2] + dz[a][0], dz[a][1]);
+    Dyz[a] = dz[a][2] - dz[a][0];
+    Szz[a] = centre(sz[a][2] + sz[a][0], sz[a][1]);
+  }
+  T Sxx = M0[2] + M0[0], jx = M0[2] - M0[0];
+  T drho = centre(Sxx, M0[1]);
+  T jy = centre(My[2] + My[0], My[1]), Sxy = My[2] - My[0];
+  T Syy = centre(Myy[2] + Myy[0], Myy[1]);
+  T jz = centre(Dz[2] + Dz[0], Dz[1]), Sxz = Dz[2] - Dz[0];
+  T Syz = centre(Dyz[2] + Dyz[0], Dyz[1]);
+  T Szzt = centre(Szz[2] + Szz[0], Szz[1]);
+  if constexpr (Scaled) {
+    const T w = T(1.0 / 216.0);
+    Sxx = Sxx * w;
+    Syy = Syy * w;
+    Szzt = Szzt * w;
+    Sxy = Sxy * w;
+    Sxz = Sxz * w;
+    Syz = Syz * w;
+    drho = drho * w;
+    jx = jx * w;
+    jy = jy * w;
+    jz = jz * w;
+  }
+  // ---- velocity, second-order central moments, relaxation
+  const T rho = T(1) + drho;
+  const T r = T(1) / rho;
+  T px = jx, py = jy, pz = jz;
+  if constexpr (Force) {
+    px += T(0.5) * Fx;
+    py += T(0.5) * Fy;
+    pz += T(0.5) * Fz;
+  }
+  const T ux = px * r, uy = py * r, uz = pz * r;
+  T vxx, vyy, vzz, vxy, vxz, vyz;
+  if constexpr (Force) {
+    vxx = Sxx + ux * (px - T(2) * jx);
+    vyy = Syy + uy * (py - T(2) * jy);
+    vzz = Szzt + uz * (pz - T(2) * jz);
+    vxy = Sxy + ux * (py - jy) - uy * jx;
+    vxz = Sxz + ux * (pz - jz) - uz * jx;
+    vyz = Syz + uy * (pz - jz) - uz * jy;
+  } else {
+    vxx = Sxx - ux * jx;
+    vyy = Syy - uy * jy;
+    vzz = Szzt - uz * jz;
+    vxy = Sxy - uy * jx;
+    vxz = Sxz - uz * jx;
+    vyz = Syz - uz * jy;
+  }
+  const T mean = (vxx + vyy + vzz) * T(1.0 / 3.0);
+  const T hr = T(0.5) * om1 * r;  // E = u^2 / 2 + D / 2, D = om1 (v - mean) / rho
+  const T Ex = T(0.5) * ux * ux + hr * (vxx - mean);
+  const T Ey = T(0.5) * uy * uy + hr * (vyy - mean);
+  const T Ez = T(0.5) * uz * uz + hr * (vzz - mean);
+  const T kxy = om1 * vxy, kxz = om1 * vxz, kyz = om1 * vyz;
+  // ---- lines along z: rho phi_z - w, kyz psi_z, kxz psi_z, kxy phi_z
+  const T zero = T(0);
+  T cz[3], rz[3], xz[3], yz[3];
+  emit_line<T, Scaled>(drho, Ez * rho, pz, cz[0], cz[1], cz[2]);
+  emit_line<T, Scaled>(zero, uz * kyz, kyz, rz[0], rz[1], rz[2]);
+  emit_line<T, Scaled>(zero, uz * kxz, kxz, xz[0], xz[1], xz[2]);
+  emit_line<T, Scaled>(kxy, Ez * kxy, uz * kxy, yz[0], yz[1], yz[2]);
+  // the force's first-order moments have no second-order part: chi = (1, 0, 0)
+  T hz[3], qz[3], Hx = zero, Hy = zero, Hz = zero;
+  if constexpr (Force) {
+    Hx = T(0.5) * ux * ux - T(1.0 / 6.0);
+    Hy = T(0.5) * uy * uy - T(1.0 / 6.0);
+    Hz = T(0.5) * uz * uz - T(1.0 / 6.0);
+    emit_line<T, Scaled>(T(1), Hz, uz, hz[0], hz[1], hz[2]);
+    const T f = T(0.5) * Fz;
+    emit_line<T, Scaled>(zero, uz * f, f, qz[0], qz[1], qz[2]);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    // ---- lines along y at this e_z
+    const T A = cz[k] + T(Scaled ? 1.0 : w1(k));
+    T cy[3], ry[3], gy[3];
+    emit_line<T, Scaled>(cz[k], Ey * A + uy * rz[k], uy * A + rz[k], cy[0], cy[1], cy[2]);
+    emit_line<T, Scaled>(xz[k], Ey * xz[k] + uy * yz[k], uy * xz[k] + yz[k], ry[0], ry[1], ry[2]);
+    if constexpr (Force) {
+      // Fx/2 chi_y chi_z joins the x lines' R; Fy/2 psi_y chi_z + Fz/2 chi_y psi_z
+      // is their chi slot
+      const T f = T(0.5) * Fx * hz[k], q = T(0.5) * Fy * hz[k];
+      T lo, mid, hi;
+      emit_line<T, Scaled>(f, Hy * f, uy * f, lo, mid, hi);
+      ry[0] += lo;
+      ry[1] += mid;
+      ry[2] += hi;
+      emit_line<T, Scaled>(qz[k], Hy * qz[k] + uy * q, uy * qz[k] + q, gy[0], gy[1], gy[2]);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      // ---- lines along x
+      const T Ax = cy[b] + T(Scaled ? 1.0 : w1(b) * w1(k));
+      T& lo = g[D3Q27::index(-1, b - 1, k - 1)];
+      T& mid = g[D3Q27::index(0, b - 1, k - 1)];
+      T& hi = g[D3Q27::index(1, b - 1, k - 1)];
+      if constexpr (Force)
+        emit_line<T, Scaled>(cy[b] + gy[b], Ex * Ax + ux * ry[b] + Hx * gy[b], ux * (Ax + gy[b]) + ry[b], lo, mid, hi);
+      else
+        emit_line<T, Scaled>(cy[b], Ex * Ax + ux * ry[b], ux * Ax + ry[b], lo, mid, hi);
+    }
+  }
+}
+
+// the form that a storage's update uses
+template <class T, bool Force, bool Scaled>
+__device__ __forceinline__ void collide27(T* g, T omega, T Fx, T Fy, T Fz) {
+  if constexpr (Scaled || std::is_same<T, double>::value) collide27_lines<T, Force, Scaled>(g, T(1) - omega, Fx, Fy, Fz);
+  else collide27_closed<T, Force>(g, omega, Fx, Fy, Fz);
 }
 
 // Product-form D3Q27 equilibrium minus the weights: the distribution whose

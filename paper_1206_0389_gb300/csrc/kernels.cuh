@@ -45,6 +45,7 @@ struct LevelPtrs {
   void* aux_dst;      // |S| per cell [nblocks][512] (real) or nullptr
   int BX, BY, BZ;     // level box in blocks
   double tau0;
+  double omega;       // 1 / tau0, rounded as the compute type divides
 };
 
 struct UpdateArgs {

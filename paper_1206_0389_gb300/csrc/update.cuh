@@ -205,9 +205,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
           const int64_t n = int64_t(L.BX) * L.BY * L.BZ * kCells;
           const int64_t j = int64_t(w.block) * kCells + c;
           const T* F = reinterpret_cast<const T*>(a.force);
-          collide27_closed<T, true, kScaled>(g, T(1) / tau0, F[j], F[n + j], F[2 * n + j]);
+          collide27<T, true, kScaled>(g, T(L.omega), F[j], F[n + j], F[2 * n + j]);
         } else {
-          collide27_closed<T, false, kScaled>(g, T(1) / tau0, T(0), T(0), T(0));
+          collide27<T, false, kScaled>(g, T(L.omega), T(0), T(0), T(0));
         }
       }
       S* q = dst + c;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
     const int dyp = (w.edges & 8) ? -BX * (L.BY - 1) : BX;
     const int dzm = (w.edges & 16) ? BXY * (L.BZ - 1) : -BXY;
     const int dzp = (w.edges & 32) ? -BXY * (L.BZ - 1) : BXY;
-    const V2 tau0 = V2(float(L.tau0), float(L.tau0));
+    const V2 tau0 = V2(float(L.tau0), float(L.tau0)), omega = V2(float(L.omega), float(L.omega));
     const S* __restrict__ src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
     S* __restrict__ dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
     auto active = [&](int c) {
@@ -355,10 +355,10 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
           const int64_t n = int64_t(L.BX) * L.BY * L.BZ * kCells;
           const int64_t j = int64_t(w.block) * kCells + c0;
           const float* F = reinterpret_cast<const float*>(a.force);
-          collide27_closed<V2, true, true>(g, V2(1.0) / tau0, V2(F[j], F[j + 1]), V2(F[n + j], F[n + j + 1]),
-                                           V2(F[2 * n + j], F[2 * n + j + 1]));
+          collide27<V2, true, true>(g, omega, V2(F[j], F[j + 1]), V2(F[n + j], F[n + j + 1]),
+                                    V2(F[2 * n + j], F[2 * n + j + 1]));
         } else {
-          collide27_closed<V2, false, true>(g, V2(1.0) / tau0, V2(0.0), V2(0.0), V2(0.0));
+          collide27<V2, false, true>(g, omega, V2(0.0), V2(0.0), V2(0.0));
         }
       }
       S* q = dst + c0;
