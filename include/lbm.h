@@ -183,7 +183,8 @@ int lbm_init_equilibrium(lbm_ctx* ctx, int level, const double* rho, const doubl
 int lbm_set_force(lbm_ctx* ctx, const double* F);
 
 /* Advance coarse_steps coarse time steps (each level l takes 2^l substeps per
- * coarse step).  Enqueues one CUDA graph per coarse step. */
+ * coarse step).  Enqueues CUDA graphs of 16 coarse steps, and of one for the
+ * rest. */
 int lbm_step(lbm_ctx* ctx, int coarse_steps);
 
 /* Wait for all enqueued work; reports launch/runtime errors. */
@@ -314,8 +315,8 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* dLdf_T, double* dLdF);
 
 /* Kernel timing: when enabled, lbm_step launches kernels directly (no graph)
  * between CUDA events on the context stream and accumulates per-kind device
- * time.  kinds: 0 update (stream-collide), 1 coarse-to-fine, 2 fine-to-coarse,
- * 3 boundary, 4 other (nothing of a step; an lbm_adjoint_backward call adds the device time of
+ * time.  kinds: 0 update (stream-collide), 1 coarse-to-fine (with the boundary
+ * ghosts and nozzle links that share its launch), 2 fine-to-coarse, 3 boundary, 4 other (nothing of a step; an lbm_adjoint_backward call adds the device time of
  * its recompute + adjoint sweep here as one entry).  ms[k] total
  * milliseconds, launches[k] launch counts. */
 int lbm_set_profiling(lbm_ctx* ctx, int enable);

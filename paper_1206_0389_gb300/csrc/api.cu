@@ -34,14 +34,12 @@ namespace {
 thread_local std::string g_create_error;
 
 struct Op {
-  enum Kind { UPDATE, C2F, F2C, BC, LINK } kind;
+  enum Kind { GHOSTS, UPDATE, F2C } kind;
   int k = 0;            // finest-level substep of the coarse step the op belongs to
-  bool level0 = false;  // an update of level-0 blocks alone (first substep of a nested grid)
+  bool level0 = false;  // level 0 alone, on the graph's branch beside the fine levels (split_level0)
+  GhostArgs ga{};
   UpdateArgs ua{};
-  C2FArgs ca{};
   F2CArgs fa{};
-  BCArgs ba{};
-  LinkArgs la{};
 };
 
 struct DevLevel {
@@ -68,10 +66,9 @@ struct lbm_ctx {
   double omega = 1.0, cs = 0.0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  // streams and events of the coarse-step graph's branches: the inflow
-  // launch beside the coarse-to-fine launch (side), and the fine-level chain
-  // (fine, high priority) beside the level-0 update (the capturing stream)
-  cudaStream_t side = nullptr, fine = nullptr;
+  // stream and events of the coarse-step graph's branches: the fine-level
+  // chain (fine, high priority) beside the level-0 update (the capturing stream)
+  cudaStream_t fine = nullptr;
   std::vector<cudaEvent_t> fork_join;
   int device = 0, sms = 1;
   bool host_direct = false;  // kernels reach ordinary host memory through the host's page tables
@@ -196,7 +193,6 @@ void free_all(lbm_ctx* c) {
   cudaFree(c->stage);
   release_adjoint(c);
   for (cudaEvent_t e : c->fork_join) cudaEventDestroy(e);
-  if (c->side) cudaStreamDestroy(c->side);
   if (c->fine) cudaStreamDestroy(c->fine);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
@@ -226,12 +222,17 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
         break;
       }
     auto sub = [&](int l) { return k / (1 << (L - 1 - l)); };
-    // coarse-to-fine for every level starting a substep: one launch (level
-    // l writes its ghost cells and reads active / hidden-1 cells of l-1)
-    if (std::max(lmin, 1) < L) {
+    // one launch for all that the levels starting a substep pull from outside
+    // their updated cells; where level 0 has a branch of its own, its part
+    // goes there
+    auto ghosts = [&](int l_lo, int l_hi, bool level0) {
       Op op;
-      op.kind = Op::C2F;
-      C2FArgs& a = op.ca;
+      op.kind = Op::GHOSTS;
+      op.k = k;
+      op.level0 = level0;
+      // coarse-to-fine (level l writes its ghost cells and reads active /
+      // hidden-1 cells of l-1)
+      C2FArgs& a = op.ga.c2f;
       a.cs2_3 = cs2_3;
       a.step = c->d_step;
       a.y0 = c->y0;
@@ -241,7 +242,7 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
       a.perturb = c->perturb;
       a.seed = c->seed;
       a.closed = c->plan.nozzle_level >= 0;
-      for (int l = std::max(lmin, 1); l < L; ++l) {
+      for (int l = std::max(l_lo, 1); l < l_hi; ++l) {
         const int s = sub(l) % 2;
         const LevelPlan& fp = c->plan.lv[l];
         const LevelPlan& cp = c->plan.lv[l - 1];
@@ -268,27 +269,19 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
         v.tau0_f = fp.tau0;
         a.n += v.n;
       }
-      if (a.n > 0) {
-        op.k = k;
-        ops.push_back(op);
-      }
-    }
-    // inflow / outflow ghosts of the same levels (after the interface: an
-    // inflow ghost may take its density from a coarse-to-fine ghost cell)
-    if (!c->plan.periodic_x) {
-      Op op;
-      op.kind = Op::BC;
-      BCArgs& b = op.ba;
+      // inflow / outlet ghosts of the same levels (an inflow ghost that takes
+      // its density from a coarse-to-fine ghost cell is written with that)
+      BCArgs& b = op.ga.bc;
       b.step = c->d_step;
       b.y0 = c->y0;
       b.z0 = c->z0;
-      b.r2 = (0.5 * c->diameter) * (0.5 * c->diameter);
+      b.r2 = a.r2;
       b.u_in = c->u_in;
       b.perturb = c->perturb;
       b.seed = c->seed;
       b.rl_out = c->rho_out - 1.0;
-      b.closed = c->plan.nozzle_level >= 0;
-      for (int l = lmin; l < L; ++l) {
+      b.closed = a.closed;
+      for (int l = l_lo; l < l_hi && !c->plan.periodic_x; ++l) {
         const LevelPlan& lp = c->plan.lv[l];
         if (lp.bc.empty()) continue;
         BCLevel& v = b.lv[b.nlv++];
@@ -301,33 +294,30 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
         v.inv_scale = std::ldexp(1.0, -l);
         b.n += v.n;
       }
-      op.k = k;
-      if (b.n > 0) ops.push_back(op);
-    }
-    // nozzle links of its level (after the level's previous update, before
-    // this one; they touch only cells near the body)
-    const int ln = c->plan.nozzle_level;
-    if (ln >= lmin && !c->plan.lv[ln].links.empty()) {
-      Op op;
-      op.kind = Op::LINK;
-      LinkArgs& a = op.la;
-      a.items = c->dl[ln].links;
-      a.n = int(c->plan.lv[ln].links.size());
-      a.f = c->dl[ln].f[par[ln]];
-      a.level = ln;
-      a.substep = sub(ln);
-      a.NY = c->plan.lv[ln].NY;
-      a.inv_scale = std::ldexp(1.0, -ln);
-      a.step = c->d_step;
-      a.y0 = c->y0;
-      a.z0 = c->z0;
-      a.r2 = (0.5 * c->diameter) * (0.5 * c->diameter);
-      a.u_in = c->u_in;
-      a.perturb = c->perturb;
-      a.seed = c->seed;
-      op.k = k;
-      ops.push_back(op);
-    }
+      // nozzle links of its level (they touch only cells near the body)
+      const int ln = c->plan.nozzle_level;
+      if (ln >= l_lo && ln < l_hi) {
+        LinkArgs& n = op.ga.link;
+        n.items = c->dl[ln].links;
+        n.n = int(c->plan.lv[ln].links.size());
+        n.f = c->dl[ln].f[par[ln]];
+        n.level = ln;
+        n.substep = sub(ln);
+        n.NY = c->plan.lv[ln].NY;
+        n.inv_scale = std::ldexp(1.0, -ln);
+        n.step = c->d_step;
+        n.y0 = c->y0;
+        n.z0 = c->z0;
+        n.r2 = a.r2;
+        n.u_in = c->u_in;
+        n.perturb = c->perturb;
+        n.seed = c->seed;
+      }
+      if (a.n > 0 || b.n > 0 || op.ga.link.n > 0) ops.push_back(op);
+    };
+    const bool branch0 = lmin == 0 && split_level0(c);
+    if (branch0) ghosts(0, 1, true);
+    ghosts(branch0 ? 1 : lmin, L, false);
     Op up;
     up.kind = Op::UPDATE;
     UpdateArgs& u = up.ua;
@@ -353,13 +343,8 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
     u.slip = c->plan.slip;
     // only the inflow reads the step counter, before the last update
     u.step_inc = k == K - 1 && !c->plan.periodic_x ? c->d_step : nullptr;
-    // a coarse step of one level without ghosts is this launch alone.  FP64
-    // storage, bound by the float64 pipes, waits for the launch to end: CTAs
-    // that come in among the last of the step before spread unevenly over the
-    // SMs (32^3 D3Q19: 16.8 us per step, chained 22.7)
-    u.chained = L == 1 && c->plan.periodic_x && c->storage != LBM_F64;
     up.k = k;
-    if (lmin == 0 && split_level0(c)) {
+    if (branch0) {
       // the first substep updates level 0 in a launch of its own: nothing
       // reads its result before the midpoint of the coarse step, so the
       // graph runs it beside the fine levels' first half
@@ -407,25 +392,35 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
   return ops;
 }
 
-cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st) {
+// Whether consecutive launches of a stream are chained (chained.cuh).  Not in
+// nested grids: the shared memory of the coarse-to-fine launch then stays
+// carved out of the L1 that the overlapping update kernels live on (2-level
+// D3Q27 FP32 jet 911 us per coarse step, chained 1079).  Not with FP64 storage:
+// bound by the float64 pipes, it suffers from CTAs that come in among the
+// last of the step before and spread unevenly over the SMs (32^3 D3Q19 16.8 us
+// per step, chained 22.7).
+bool chain_launches(const lbm_ctx* c) { return c->L == 1 && c->storage != LBM_F64; }
+
+cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st, bool chained = false) {
   switch (op.kind) {
-    case Op::UPDATE: return launch_update(c->model, c->storage, op.ua, c->threads, c->minb, c->ctas, st);
-    case Op::C2F: return launch_c2f(c->model, c->storage, op.ca, st);
+    case Op::GHOSTS: return launch_ghosts(c->model, c->storage, op.ga, chained, st);
+    case Op::UPDATE: {
+      UpdateArgs a = op.ua;
+      a.chained = chained;
+      return launch_update(c->model, c->storage, a, c->threads, c->minb, c->ctas, st);
+    }
     case Op::F2C: return launch_f2c(c->model, c->storage, op.fa, st);
-    case Op::BC: return launch_bc(c->model, c->storage, op.ba, st);
-    case Op::LINK: return launch_links(c->model, c->storage, op.la, st);
   }
   return cudaErrorInvalidValue;
 }
-cudaError_t run_op(lbm_ctx* c, const Op& op) { return run_op(c, op, c->stream); }
 
+// kinds of lbm_get_profile (a launch of several kinds of ghosts counts as
+// coarse-to-fine)
 int op_kind_index(const Op& op) {
   switch (op.kind) {
+    case Op::GHOSTS: return op.ga.c2f.n > 0 ? 1 : 3;
     case Op::UPDATE: return 0;
-    case Op::C2F: return 1;
     case Op::F2C: return 2;
-    case Op::BC:
-    case Op::LINK: return 3;
   }
   return 4;
 }
@@ -457,7 +452,7 @@ int restrict_all(lbm_ctx* ctx) {
 // Short coarse steps (small grids) are bound by the launch of a graph per
 // step, so a run of steps goes out as graphs of kManySteps steps: 53,760 cells
 // of D3Q27 FP32 8.4 -> 4.4 us per step, 96^3 36.9 -> 31.3, 256^3 FP16 309 -> 300
-// (with the chained launches of begin_update).  The number is even: the parity comes round.
+// (with chained launches).  The number is even: the parity comes round.
 constexpr int kManySteps = 16;
 
 // captures `steps` coarse steps that start at level-0 parity p0
@@ -475,52 +470,35 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
       return cudaSuccess;
     };
     // Nested FP16 grids: the chain of ops runs on the high-priority stream `fine`;
-    // the level-0 update of the first substep runs on the capturing stream
-    // beside it, after the level-0 inflow (and nozzle links) it reads, and
-    // joins the chain before the first op of the second half of the coarse
-    // step (the coarse-to-fine launch that reads level 0's new state, the
-    // restriction into level 0); that restriction in turn runs beside the
-    // rest of the chain (nothing after it touches level 0).  The level-0
-    // blocks fill the SMs the short interface launches leave idle.
+    // level 0's ghosts and update of the first substep run on the capturing
+    // stream beside it and join the chain before the first op of the second
+    // half of the coarse step (the coarse-to-fine launch that reads level 0's
+    // new state, the restriction into level 0); that restriction in turn runs
+    // beside the rest of the chain (nothing after it touches level 0).  The
+    // level-0 blocks fill the SMs the short interface launches leave idle.
     const bool split = split_level0(ctx);
     cudaStream_t st = ctx->stream;
-    cudaEvent_t u0_after = nullptr, u0_done = nullptr, r0_done = nullptr, evt = nullptr;
+    cudaEvent_t u0_done = nullptr, r0_done = nullptr, evt = nullptr;
     if (split) {
       if ((e = next_event(&evt)) == cudaSuccess && (e = cudaEventRecord(evt, ctx->stream)) == cudaSuccess)
         e = cudaStreamWaitEvent(ctx->fine, evt, 0);
       st = ctx->fine;
     }
+    const bool chain = chain_launches(ctx);
     for (size_t k = 0; k < ops.size() && e == cudaSuccess; ++k) {
       const Op& op = ops[k];
       if (u0_done && op.k >= K / 2) {
         if ((e = cudaStreamWaitEvent(st, u0_done, 0)) != cudaSuccess) break;
         u0_done = nullptr;
       }
-      // the inflow launch after a coarse-to-fine launch touches other cells
-      // (inflow ghosts fed by ghost cells are written by the latter), so the
-      // graph runs the two side by side
-      if (op.kind == Op::C2F && k + 1 < ops.size() && ops[k + 1].kind == Op::BC) {
-        cudaEvent_t fork = nullptr, join = nullptr;
-        if ((e = next_event(&fork)) != cudaSuccess || (e = next_event(&join)) != cudaSuccess ||
-            (e = cudaEventRecord(fork, st)) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(ctx->side, fork, 0)) != cudaSuccess ||
-            (e = run_op(ctx, ops[k + 1], ctx->side)) != cudaSuccess ||
-            (e = run_op(ctx, op, st)) != cudaSuccess ||
-            (e = cudaEventRecord(join, ctx->side)) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess)
-          break;
-        if (ops[k + 1].k == 0) u0_after = join;  // the inflow is done
-        ++k;
-        continue;
-      }
-      if (split && op.level0 && op.kind == Op::UPDATE) {
-        if (u0_after && (e = cudaStreamWaitEvent(ctx->stream, u0_after, 0)) != cudaSuccess) break;
-        if ((e = run_op(ctx, op, ctx->stream)) != cudaSuccess || (e = next_event(&u0_done)) != cudaSuccess ||
-            (e = cudaEventRecord(u0_done, ctx->stream)) != cudaSuccess)
+      if (op.level0 && op.kind != Op::F2C) {
+        if ((e = run_op(ctx, op, ctx->stream)) != cudaSuccess) break;
+        if (op.kind == Op::UPDATE && ((e = next_event(&u0_done)) != cudaSuccess ||
+                                      (e = cudaEventRecord(u0_done, ctx->stream)) != cudaSuccess))
           break;
         continue;
       }
-      if (split && op.level0 && op.kind == Op::F2C && !u0_done && !r0_done) {
+      if (op.level0 && !u0_done && !r0_done) {
         // after the chain so far; joined at the end of the coarse step
         cudaEvent_t here = nullptr;
         if ((e = next_event(&here)) != cudaSuccess || (e = cudaEventRecord(here, st)) != cudaSuccess ||
@@ -530,11 +508,7 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
           break;
         continue;
       }
-      if ((e = run_op(ctx, op, st)) != cudaSuccess) break;
-      if (split && op.k == 0 && (op.kind == Op::BC || (op.kind == Op::LINK && op.la.level == 0))) {
-        // the level-0 update waits for the chain up to here
-        if ((e = next_event(&u0_after)) != cudaSuccess || (e = cudaEventRecord(u0_after, st)) != cudaSuccess) break;
-      }
+      if ((e = run_op(ctx, op, st, chain && (s > 0 || k > 0))) != cudaSuccess) break;
     }
     if (split && e == cudaSuccess) {
       if (u0_done) e = cudaStreamWaitEvent(st, u0_done, 0);
@@ -582,6 +556,7 @@ int autotune(lbm_ctx* ctx) {
   if (!big || big->ua.nitems == 0) return LBM_OK;
   UpdateArgs trial = big->ua;
   trial.step_inc = nullptr;
+  trial.chained = chain_launches(ctx);
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -923,13 +898,12 @@ int create_context(lbm_ctx** out, lbm_model model, lbm_storage storage, const lb
     // stream priority, the level-0 update beside it at the caller's
     int least = 0, greatest = 0;
     ce = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest);
     if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ctx->fine, cudaStreamNonBlocking, greatest);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(ce));
   }
-  // events of one coarse-step capture: a fork and a join per coarse-to-fine
-  // launch, and at most six for the level-0 branches
-  ctx->fork_join.assign(2 * (1 << (ctx->L - 1)) + 8, nullptr);
+  // events of one coarse step's branches: the fork, level 0 updated, the
+  // restriction's fork and join, the end
+  ctx->fork_join.assign(5, nullptr);
   for (cudaEvent_t& e : ctx->fork_join) {
     ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("event: ") + cudaGetErrorString(ce));
@@ -1118,7 +1092,7 @@ int lbm_step(lbm_ctx* ctx, int coarse_steps) {
       std::vector<Op> ops = build_schedule(ctx, ctx->parity0);
       for (const Op& op : ops) {
         CK(cudaEventRecord(e0, ctx->stream));
-        CK(run_op(ctx, op));
+        CK(run_op(ctx, op, ctx->stream));
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaEventSynchronize(e1));
         float ms = 0;
@@ -1596,6 +1570,7 @@ int lbm_adjoint_forward(lbm_ctx* ctx, int T, int checkpoint_every) {
     UpdateArgs ua{};
     for (const Op& op : ops)
       if (op.kind == Op::UPDATE) ua = op.ua;
+    ua.chained = chain_launches(ctx);
     CK(cudaMemcpyAsync(ctx->adj_ck[0], ctx->dl[0].f[ctx->parity0], sb, cudaMemcpyDeviceToDevice, ctx->stream));
     for (int t = 0; t < T; ++t) {
       ua.lv[0].src = ctx->adj_ck[t];

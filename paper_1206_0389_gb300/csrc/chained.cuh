@@ -1,0 +1,30 @@
+// Programmatic dependent launches: a chained launch is set up, down to resident
+// CTAs, while the kernel before it in the stream drains.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace lbm {
+
+// First statement of a kernel that may be chained: lets the next launch come
+// up, and holds every thread until the kernel before has ended and its writes
+// are visible (a launch without the attribute passes at once).
+__device__ __forceinline__ void begin_chained() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class Args>
+cudaError_t launch_chained(void (*kernel)(const Args), int grid, int tpb, const Args& a, bool chained, cudaStream_t st) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(grid));
+  cfg.blockDim = dim3(unsigned(tpb));
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+}  // namespace lbm

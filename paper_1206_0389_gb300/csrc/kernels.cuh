@@ -66,8 +66,8 @@ struct UpdateArgs {
                           // of one CTA (set by the launcher)
   long long* step_inc;    // coarse-step counter that the last update of a coarse step
                           // advances (nothing after it in the step reads it), or nullptr
-  int chained;            // the launch may begin while the launch before it, an update
-                          // too, still ends (programmatic dependent launch)
+  int chained;            // the launch may begin while the kernel before it still ends
+                          // (chained.cuh)
   int run_mask;           // cells (FP16 pairs) per run - 1 (set by the launcher)
 };
 
@@ -223,15 +223,20 @@ struct LinkArgs {
   unsigned long long seed;
 };
 
+// what one launch brings in before an update (parts with n = 0 are absent)
+struct GhostArgs {
+  C2FArgs c2f;
+  BCArgs bc;
+  LinkArgs link;
+};
+
 // ------------------------------------------------------------------ launchers
 // model: 0 D3Q19 MRT-LES, 1 D3Q27 FCLB; storage: lbm_storage.
 cudaError_t launch_update(int model, int storage, const UpdateArgs& a, int threads, int minb, int ctas,
                           cudaStream_t st);
 cudaError_t update_occupancy(int model, int storage, bool walls, int threads, int minb, int* ctas_per_sm);
-cudaError_t launch_c2f(int model, int storage, const C2FArgs& a, cudaStream_t st);
+cudaError_t launch_ghosts(int model, int storage, const GhostArgs& a, bool chained, cudaStream_t st);
 cudaError_t launch_f2c(int model, int storage, const F2CArgs& a, cudaStream_t st);
-cudaError_t launch_bc(int model, int storage, const BCArgs& a, cudaStream_t st);
-cudaError_t launch_links(int model, int storage, const LinkArgs& a, cudaStream_t st);
 
 // dense <-> block staging for one slab of cell layers [z0, z0 + nz) of a level
 enum SlabMode { SLAB_SET_STATE = 0, SLAB_GET_STATE = 1, SLAB_INIT_EQ = 2, SLAB_MACRO = 3,

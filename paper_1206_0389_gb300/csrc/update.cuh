@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "chained.cuh"
 #include "collide.cuh"
 #include "kernels.cuh"
 #include "pair.cuh"
@@ -50,14 +51,10 @@ __device__ __forceinline__ float ldg_f32_l2(const float* p) {
   return v;
 }
 
-// Start of an update kernel.  A chained launch (a.chained) is set up, down to
-// resident CTAs, while the update before it drains; griddepcontrol.wait holds
-// every thread until that one has ended and its writes are visible (a launch
-// without the attribute passes at once).  With the graphs of 16 steps: 96^3
+// Start of an update kernel (chained.cuh).  With the graphs of 16 steps: 96^3
 // D3Q27 FP32 36.9 -> 31.3 us per step, 256^3 520 -> 515 us.
 __device__ __forceinline__ void begin_update(const UpdateArgs& a) {
-  asm volatile("griddepcontrol.launch_dependents;");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  begin_chained();
   if (a.step_inc != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *a.step_inc += 1;
 }
 
@@ -400,20 +397,6 @@ inline int split_for(int nitems, int max_runs, int resident, bool always) {
 }
 
 template <class K>
-cudaError_t launch_chained(K kernel, int grid, int tpb, const UpdateArgs& a, cudaStream_t st) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(unsigned(tpb));
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = a.chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-template <class K>
 cudaError_t resident_ctas(K kernel, int tpb, int& occ, int* resident) {
   cudaError_t e = cudaSuccess;
   if (occ == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, tpb, 0);
@@ -438,7 +421,7 @@ cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   // wait longer in L2) or the grid (persistent CTAs take items grid apart);
   // a list short enough to be split is resident as a whole
   a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : resident / 2;
-  return launch_chained(k_update_pair<M, TPB, MINB>, grid, TPB, a, st);
+  return launch_chained(k_update_pair<M, TPB, MINB>, grid, TPB, a, a.chained, st);
 }
 template <class M>
 cudaError_t launch_pair(const UpdateArgs& a, int threads, int minb, int ctas, cudaStream_t st) {
@@ -468,7 +451,7 @@ cudaError_t launch_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   a.split = split_for(a.nitems, kCells / TPB, resident, std::is_same<S, double>::value);
   a.run_mask = (kCells >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
-  return launch_chained(k_update<M, S, TPB, MINB, W>, grid, TPB, a, st);
+  return launch_chained(k_update<M, S, TPB, MINB, W>, grid, TPB, a, a.chained, st);
 }
 
 template <class M, class S, bool W>
