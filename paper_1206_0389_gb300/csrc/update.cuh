@@ -65,21 +65,6 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
   using T = typename St::T;
   constexpr int Q = M::Q;
   constexpr int QS = Q * kCells;
-  // FP16 storage holds (f_i - w_i) / w_i: the collision takes and returns
-  // that form directly (the weights fold into its constants)
-  constexpr bool kScaled = std::is_same<S, __half>::value;
-  // FP16 D3Q19 prefetches the next cell (fits in 64 registers; measured
-  // 0.79 -> 0.81 of the copy peak); the D3Q27 collision has no registers to
-  // spare for it (the prefetch spills and runs 25 % slower)
-  constexpr bool kPipeline = kScaled && Q == 19;
-  // FP16 D3Q27 instead prefetches the next cells into L2 (0.78 -> 0.80 of
-  // the copy peak; on the FP32 kernels, already HBM-bound, it gained nothing)
-  constexpr bool kPrefetch = kScaled && !kPipeline;
-  const int pf_lane = threadIdx.x & 31;  // the population this lane prefetches
-  int pf_shift = 0;                      // its in-block pull shift e_x + 8 e_y + 64 e_z
-  static_for<Q>([&](auto i) {
-    if (pf_lane == int(i)) pf_shift = Lattice<Q>::ex(i) + 8 * Lattice<Q>::ey(i) + 64 * Lattice<Q>::ez(i);
-  });
   // a unit of work is one of 2^split equal runs of a block's cells
   // (a.run_mask = cells per run - 1; a thread ends its run when its cell
   // index wraps to the run's first TPB cells, which needs no register for
@@ -187,78 +172,42 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
             else if (cy && cz) q = p + (iyz * kCells - ex + X);
             else if (cy) q = (ez == 1 ? b1 : ez == -1 ? bm : p) + (iy * kCells - (ex + 64 * ez) + X);
             else q = p + (iz * kCells - (ex + 8 * ey) + X + Y);
-            if constexpr (kScaled) g[i] = __half2float(__ldg(q));
-            else g[i] = St::template get<Q, i>(q);
+            g[i] = St::template get<Q, i>(q);
           }
         }
       });
     };
     auto collide_store = [&](int c, T (&g)[Q]) {
       if constexpr (Q == 19) {
-        const T S_ = collide19<T, kScaled>(g, tau0, T(a.cs2_18));
+        const T S_ = collide19<T>(g, tau0, T(a.cs2_18));
         if (L.aux_dst) reinterpret_cast<T*>(L.aux_dst)[int64_t(w.block) * kCells + c] = S_;
       } else {
         if (a.force != nullptr && w.level == 0) {
           const int64_t n = int64_t(L.BX) * L.BY * L.BZ * kCells;
           const int64_t j = int64_t(w.block) * kCells + c;
           const T* F = reinterpret_cast<const T*>(a.force);
-          collide27<T, true, kScaled>(g, T(L.omega), F[j], F[n + j], F[2 * n + j]);
+          collide27<T, true, false>(g, T(L.omega), F[j], F[n + j], F[2 * n + j]);
         } else {
-          collide27<T, false, kScaled>(g, T(L.omega), T(0), T(0), T(0));
+          collide27<T, false, false>(g, T(L.omega), T(0), T(0), T(0));
         }
       }
       S* q = dst + c;
-      static_for<Q>([&](auto i) {
-        if constexpr (kScaled) q[int(i) * kCells] = __float2half_rn(g[i]);
-        else St::template put<Q, i>(q + int(i) * kCells, g[i]);
-      });
+      static_for<Q>([&](auto i) { St::template put<Q, i>(q + int(i) * kCells, g[i]); });
     };
-    if constexpr (kPipeline) {
-      // half-size loads keep half the bytes in flight, so the raw values of
-      // the thread's next cell are loaded while this one collides
-      __half cur[Q], nxt[Q];
-      pull(c0, [&](auto i, const S* p) { cur[i] = __ldg(p); });
-      int c = c0;
+    int c = c0;
 #pragma unroll 1
-      do {
-        if (((c + TPB) & a.run_mask) >= TPB) pull(c + TPB, [&](auto i, const S* p) { nxt[i] = __ldg(p); });
-        if (active(c)) {
-          T g[Q];
-          static_for<Q>([&](auto i) { g[i] = __half2float(cur[i]); });
-          if constexpr (W) if (wf) wall_fix(c, g);
-          collide_store(c, g);
-        }
-        static_for<Q>([&](auto i) { cur[i] = nxt[i]; });
-        c += TPB;
-      } while ((c & a.run_mask) >= TPB);
-    } else {
-      int c = c0;
-#pragma unroll 1
-      do {
-        if constexpr (kPrefetch) {
-          // the warp's next cells in this block: lane q asks L2 for the run
-          // of population q they pull (one instruction per warp, no
-          // registers held), so the next loads wait on L2, not DRAM
-          const int cn = (c & ~31) + TPB;
-          if (pf_lane < Q && (cn & a.run_mask) >= TPB) {
-            int sc = cn - pf_shift;
-            sc = sc < 0 ? 0 : sc > kCells - 1 ? kCells - 1 : sc;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(src + pf_lane * kCells + sc));
-          }
-        }
-        if (active(c)) {
-          T g[Q];
-          pull(c, [&](auto i, const S* p) {
-            if constexpr (kScaled) g[i] = __half2float(ldg_half_l2(p));
-            else if constexpr (std::is_same<S, float>::value) g[i] = ldg_f32_l2(p);
-            else g[i] = St::template get<Q, i>(p);
-          });
-          if constexpr (W) if (wf) wall_fix(c, g);
-          collide_store(c, g);
-        }
-        c += TPB;
-      } while ((c & a.run_mask) >= TPB);
-    }
+    do {
+      if (active(c)) {
+        T g[Q];
+        pull(c, [&](auto i, const S* p) {
+          if constexpr (std::is_same<S, float>::value) g[i] = ldg_f32_l2(p);
+          else g[i] = St::template get<Q, i>(p);
+        });
+        if constexpr (W) if (wf) wall_fix(c, g);
+        collide_store(c, g);
+      }
+      c += TPB;
+    } while ((c & a.run_mask) >= TPB);
   }
 }
 
@@ -269,8 +218,11 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
 // with e_x = 0 come in as one aligned half2 load for both cells, and every
 // population leaves as one half2 store.  Pulls with e_x != 0 are two scalar
 // loads (their sources straddle the pair alignment).  Mixed pairs (one cell
-// masked out) store only the active cell.
-template <class M, int TPB, int MINB>
+// masked out) store only the active cell.  Storage holds (f_i - w_i) / w_i,
+// which the collision takes and returns.  W = true: walls as in k_update; both
+// cells of a pair share their y and z faces, an x face has one of them.
+// 192 x 80 x 112 D3Q19 with walls: 27.7 us per step (a cell per thread: 33.2).
+template <class M, int TPB, int MINB, bool W>
 __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
   using S = __half;
   constexpr int Q = M::Q;
@@ -297,6 +249,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
     const int dyp = (w.edges & 8) ? -BX * (L.BY - 1) : BX;
     const int dzm = (w.edges & 16) ? BXY * (L.BZ - 1) : -BXY;
     const int dzp = (w.edges & 32) ? -BXY * (L.BZ - 1) : BXY;
+    const int wf = (W && w.level == 0)
+                       ? (a.walls & (((w.edges >> 2) & 15) | ((w.edges & 128) ? 16 : 0) | ((w.edges & 64) ? 32 : 0)))
+                       : 0;  // as in k_update
     const V2 tau0 = V2(float(L.tau0), float(L.tau0)), omega = V2(float(L.omega), float(L.omega));
     const S* __restrict__ src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
     S* __restrict__ dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
@@ -340,6 +295,42 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
           g[i] = V2(__half2float(ldg_half_l2(b + o + k)), __half2float(ldg_half_l2(b + o + k + 1 + Xp1)));
         }
       });
+      if constexpr (W) {
+        const bool yl = (wf & 1) && y == 0, yh = (wf & 2) && y == 7;
+        const bool zl = (wf & 4) && z == 0, zh = (wf & 8) && z == 7;
+        const bool xl = (wf & 16) && x0 == 0, xh = (wf & 32) && x0 == 6;
+        if (yl || yh || zl || zh || xl || xh) {
+          static_for<Q>([&](auto i) {
+            constexpr int ex = Lattice<Q>::ex(i), ey = Lattice<Q>::ey(i), ez = Lattice<Q>::ez(i);
+            if constexpr (ex != 0 || ey != 0 || ez != 0) {
+              const bool cy = ey == 1 ? yl : ey == -1 ? yh : false;
+              const bool cz = ez == 1 ? zl : ez == -1 ? zh : false;
+              const bool cx = ex == 1 ? xl : ex == -1 ? xh : false;  // of the one cell at the x face
+              if (cy || cz || cx) {
+                const bool sy = a.slip & (ey == 1 ? 1 : 2), sz = a.slip & (ez == 1 ? 4 : 8);
+                constexpr int ib = Lattice<Q>::index(-ex, -ey, -ez);
+                constexpr int iy = Lattice<Q>::index(ex, -ey, ez);
+                constexpr int iz = Lattice<Q>::index(ex, ey, -ez);
+                constexpr int iyz = Lattice<Q>::index(ex, -ey, -ez);
+                const __half2 back = __ldg(reinterpret_cast<const __half2*>(p0 + ib * kCells));
+                V2 v = g[i];
+                if ((cy && !sy) || (cz && !sz)) {
+                  v = V2(__low2float(back), __high2float(back));
+                } else if (cy || cz) {
+                  const S* q;
+                  if (cy && cz) q = p0 + (iyz * kCells - ex);
+                  else if (cy) q = (ez == 1 ? b1 : ez == -1 ? bm : p0) + (iy * kCells - (ex + 64 * ez));
+                  else q = p0 + (iz * kCells - (ex + 8 * ey) + (ey == 1 ? Ym : ey == -1 ? Yp : 0));
+                  v = V2(__half2float(__ldg(q + (ex == 1 ? Xm0 : 0))), __half2float(__ldg(q + 1 + (ex == -1 ? Xp1 : 0))));
+                }
+                if (cx && ex == 1) v.x = __low2float(back);
+                if (cx && ex == -1) v.y = __high2float(back);
+                g[i] = v;
+              }
+            }
+          });
+        }
+      }
       if constexpr (Q == 19) {
         const V2 S_ = collide19<V2, true>(g, tau0, V2(float(a.cs2_18), float(a.cs2_18)));
         if (L.aux_dst) {
@@ -375,11 +366,11 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
 }
 
 // Launch shapes the autotuner chooses from: threads per CTA, and a minimum
-// number of resident CTAs per SM that caps the registers (higher occupancy
-// for the FP16 variants, whose half-size loads keep fewer bytes in flight).
-// FP16 storage without walls runs the cell-pair kernel; a listed shape maps
-// onto it with half the minimum CTAs per SM (two cells per thread hold about
-// twice the registers): (128,1) (256,1) (128,4) (256,2) (128,5).
+// number of resident CTAs per SM that caps the registers (higher occupancy).
+// FP16 storage runs the cell-pair kernel, whose bytes in flight come from its
+// residency: D3Q19 takes the listed caps as they are (256^3, 8 CTAs of 64
+// registers: 193 us per step, 7: 198, 6: 203, 5: 217), D3Q27 keeps 6, 5 or 3
+// (6 CTAs of 78 registers: 286 us; 7: 289, and with walls it spills).
 
 // Splitting the blocks of short work lists: a launch with fewer blocks than
 // the part holds CTAs leaves SMs idle (64 blocks of a 32^3 grid on 152 SMs)
@@ -407,38 +398,45 @@ cudaError_t resident_ctas(K kernel, int tpb, int& occ, int* resident) {
   return e;
 }
 
-template <class M, int TPB, int MINB>
+// CTAs per SM that the cell-pair kernel is compiled for in place of a listed
+// shape's
+template <class M>
+constexpr int pair_ctas(int listed) {
+  return M::Q == 19 ? listed : listed == 8 ? 6 : listed == 7 ? 5 : 3;
+}
+template <class M, bool W, int TPB, int MINB>
 cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   static int occ = 0;  // CTAs per SM of this instance (a property of the kernel)
   int resident = 0;
-  cudaError_t e = resident_ctas(k_update_pair<M, TPB, MINB>, TPB, occ, &resident);
+  cudaError_t e = resident_ctas(k_update_pair<M, TPB, MINB, W>, TPB, occ, &resident);
   if (e != cudaSuccess) return e;
   a.split = split_for(a.nitems, kCells / 2 / TPB, resident, false);
   a.run_mask = ((kCells / 2) >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
-  // prefetch distance: half the CTAs resident at once (one CTA per block:
-  // measured better than one or two full waves, whose prefetched blocks
-  // wait longer in L2) or the grid (persistent CTAs take items grid apart);
-  // a list short enough to be split is resident as a whole
-  a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : resident / 2;
-  return launch_chained(k_update_pair<M, TPB, MINB>, grid, TPB, a, a.chained, st);
+  // prefetch distance: three eighths of the CTAs resident at once (one CTA per
+  // block: 256^3 D3Q27 285.7 us per step, a half 288, a quarter 285, none
+  // 307, all 319; D3Q19 202.9, 202.6, 205.6, 229, 204 at 6 CTAs) or the grid
+  // (persistent CTAs take items grid apart); a list short enough to be split
+  // is resident as a whole
+  a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : resident * 3 / 8;
+  return launch_chained(k_update_pair<M, TPB, MINB, W>, grid, TPB, a, a.chained, st);
 }
-template <class M>
+template <class M, bool W>
 cudaError_t launch_pair(const UpdateArgs& a, int threads, int minb, int ctas, cudaStream_t st) {
-  if (threads == 128 && minb == 7) return launch_pair_shape<M, 128, 5>(a, ctas, st);
-  if (threads == 128 && minb == 1) return launch_pair_shape<M, 128, 1>(a, ctas, st);
-  if (threads == 256 && minb == 1) return launch_pair_shape<M, 256, 1>(a, ctas, st);
-  if (threads == 128 && minb == 8) return launch_pair_shape<M, 128, 4>(a, ctas, st);
-  if (threads == 256 && minb == 4) return launch_pair_shape<M, 256, 2>(a, ctas, st);
+  if (threads == 128 && minb == 7) return launch_pair_shape<M, W, 128, pair_ctas<M>(7)>(a, ctas, st);
+  if (threads == 128 && minb == 1) return launch_pair_shape<M, W, 128, 1>(a, ctas, st);
+  if (threads == 256 && minb == 1) return launch_pair_shape<M, W, 256, 1>(a, ctas, st);
+  if (threads == 128 && minb == 8) return launch_pair_shape<M, W, 128, pair_ctas<M>(8)>(a, ctas, st);
+  if (threads == 256 && minb == 4) return launch_pair_shape<M, W, 256, pair_ctas<M>(4)>(a, ctas, st);
   return cudaErrorInvalidValue;
 }
-template <class M>
+template <class M, bool W>
 cudaError_t occ_pair(int threads, int minb, int* n) {
-  if (threads == 128 && minb == 7) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, 5>, 128, 0);
-  if (threads == 128 && minb == 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, 1>, 128, 0);
-  if (threads == 256 && minb == 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 256, 1>, 256, 0);
-  if (threads == 128 && minb == 8) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, 4>, 128, 0);
-  if (threads == 256 && minb == 4) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 256, 2>, 256, 0);
+  if (threads == 128 && minb == 7) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, pair_ctas<M>(7), W>, 128, 0);
+  if (threads == 128 && minb == 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, 1, W>, 128, 0);
+  if (threads == 256 && minb == 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 256, 1, W>, 256, 0);
+  if (threads == 128 && minb == 8) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 128, pair_ctas<M>(8), W>, 128, 0);
+  if (threads == 256 && minb == 4) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update_pair<M, 256, pair_ctas<M>(4), W>, 256, 0);
   return cudaErrorInvalidValue;
 }
 
@@ -457,8 +455,8 @@ cudaError_t launch_shape(UpdateArgs a, int ctas, cudaStream_t st) {
 template <class M, class S, bool W>
 cudaError_t launch_ms(const UpdateArgs& a, int threads, int minb, int ctas, cudaStream_t st) {
   if (a.nitems == 0) return cudaSuccess;
-  if constexpr (std::is_same<S, __half>::value && !W) {
-    return launch_pair<M>(a, threads, minb, ctas, st);
+  if constexpr (std::is_same<S, __half>::value) {
+    return launch_pair<M, W>(a, threads, minb, ctas, st);
   } else {
     if (threads == 128 && minb == 7) return launch_shape<M, S, W, 128, 7>(a, ctas, st);
     if (threads == 128 && minb == 1) return launch_shape<M, S, W, 128, 1>(a, ctas, st);
@@ -471,8 +469,8 @@ cudaError_t launch_ms(const UpdateArgs& a, int threads, int minb, int ctas, cuda
 
 template <class M, class S, bool W>
 cudaError_t occ_ms(int threads, int minb, int* n) {
-  if constexpr (std::is_same<S, __half>::value && !W) {
-    return occ_pair<M>(threads, minb, n);
+  if constexpr (std::is_same<S, __half>::value) {
+    return occ_pair<M, W>(threads, minb, n);
   } else {
     if (threads == 128 && minb == 7) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update<M, S, 128, 7, W>, 128, 0);
     if (threads == 128 && minb == 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_update<M, S, 128, 1, W>, 128, 0);
