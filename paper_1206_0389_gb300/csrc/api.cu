@@ -129,8 +129,8 @@ int cuda_fail(lbm_ctx* c, cudaError_t e, const char* where) {
 // Short results (audits, probed cells) are written by their kernel into
 // registered memory and copied out by the host: no staging copies, and no
 // first touch of the caller's pages over the link (16 probed cells of a small
-// grid: 42 us a call by pageable copies, 52-57 us written in place, 30 us so;
-// an audit 90 -> 56 us).
+// grid: 42 us a call by pageable copies, 52-57 us written in place, 17 us so,
+// with a thread per value; an audit 90 -> 56 us).
 constexpr size_t kPinBytes = size_t(64) << 10;
 
 size_t real_bytes(int storage) { return storage == LBM_F64 ? 8 : 4; }
@@ -655,9 +655,15 @@ bool bring_in(const void* p, size_t bytes, bool write) {
   const uintptr_t lo = uintptr_t(p) / page * page, hi = (uintptr_t(p) + bytes + page - 1) / page * page;
   const int advice = write ? MADV_POPULATE_WRITE : MADV_POPULATE_READ;
   auto part = [=](uintptr_t a, uintptr_t b) { return a >= b || madvise(reinterpret_cast<void*>(a), b - a, advice) == 0; };
+  // Threads: the faults of one process contend, so a few are best (1.9 GB of
+  // fresh arrays through lbm_stats_get: 1 thread 72 ms, 4 37, 8 52, 16 63), and
+  // on pages that are there already one is (13 ms, several 20), as the last
+  // page tells.
   constexpr size_t kShare = size_t(16) << 20;  // bytes worth a thread of its own
-  constexpr int kMaxThreads = 8;
-  const int n = int(std::min<size_t>({size_t(kMaxThreads), (hi - lo) / kShare + 1,
+  constexpr int kMaxThreads = 4;
+  unsigned char there = 0;
+  const bool touched = mincore(reinterpret_cast<void*>(hi - page), page, &there) == 0 && (there & 1);
+  const int n = touched ? 1 : int(std::min<size_t>({size_t(kMaxThreads), (hi - lo) / kShare + 1,
                                       size_t(std::max(1u, std::thread::hardware_concurrency()))}));
   const size_t share = ((hi - lo) / n + page - 1) / page * page;
   std::thread th[kMaxThreads];

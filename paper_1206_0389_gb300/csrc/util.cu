@@ -256,11 +256,14 @@ __global__ void k_slab(const SlabArgs a) {
   }
 }
 
+// one thread per (cell, population): a thread per cell chained Q loads of a
+// few cells one after the other, and its results lay Q apart
 template <class M, class S>
 __global__ void k_gather(const GatherArgs a) {
   constexpr int Q = M::Q;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t o = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, t = o / Q;
   if (t >= a.n) return;
+  const int i = int(o - t * Q);
   const long long c = a.cells[t];
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   const long long ncell = (long long)a.NX * a.NY * a.NZ;
@@ -269,9 +272,12 @@ __global__ void k_gather(const GatherArgs a) {
     const int x = int(c % a.NX), y = int((c / a.NX) % a.NY), z = int(c / ((long long)a.NX * a.NY));
     j = box_index(x, y, z, a.ox, a.oy, a.oz, a.BX, a.BY, a.BZ);
   }
-  const S* f = reinterpret_cast<const S*>(a.f) + (j >= 0 ? (j / kCells) * Q * kCells + j % kCells : 0);
-  for (int i = 0; i < Q; ++i)
-    a.out[t * Q + i] = j < 0 ? nan : double(load_rt<S, Q>(f + i * kCells, i)) + shift_of<Q>(i);
+  if (j < 0) {
+    a.out[o] = nan;
+    return;
+  }
+  const S* f = reinterpret_cast<const S*>(a.f) + ((j / kCells) * Q + i) * kCells + j % kCells;
+  a.out[o] = double(load_rt<S, Q>(f, i)) + shift_of<Q>(i);
 }
 
 // Float64 sums over active cells: (delta rho, j_x, j_y, j_z) times vol.
@@ -418,7 +424,7 @@ static cudaError_t slab_ms(const SlabArgs& a, cudaStream_t st) {
 template <class M, class S>
 static cudaError_t gather_ms(const GatherArgs& a, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
-  k_gather<M, S><<<unsigned((a.n + 255) / 256), 256, 0, st>>>(a);
+  k_gather<M, S><<<unsigned((a.n * M::Q + 127) / 128), 128, 0, st>>>(a);
   return cudaGetLastError();
 }
 template <class M, class S>
