@@ -199,47 +199,8 @@ __device__ __forceinline__ T collide19(T* g, T tau0, T cs2_18) {
 }
 
 // ------------------------------------------------------------------ D3Q27 FCLB
-// Central moments by three one-dimensional passes (z, then y, then x): the
-// D3Q27 velocity set is the product {-1,0,1}^3 and the central-moment
-// matrix of Section 2 factorises into 3x3 per-axis transforms.  Each pass is
-// written for deviations from the weight part: a line whose weight part is
-// K (w1(-1), w1(0), w1(+1)) = K (1/6, 2/3, 1/6) has moments K (1, 0, 1/3) at
-// rest, and the pass outputs the deviations from those.  After three passes
-// v[a][b][c] = rho kappa_abc - C_abc with C_abc = c_a c_b c_c, c = (1, 0, 1/3).
-// (Index 0/1/2 means velocity -1/0/+1 before a pass and order 0/1/2 after.)
+// one-dimensional weights (index 0/1/2 means velocity -1/0/+1)
 __host__ __device__ constexpr double w1(int k) { return k == 1 ? 2.0 / 3.0 : 1.0 / 6.0; }
-__host__ __device__ constexpr double c1(int k) { return k == 0 ? 1.0 : k == 1 ? 0.0 : 1.0 / 3.0; }
-
-template <class T>
-__device__ __forceinline__ void fwd_line(T& a, T& b, T& c, T u, T uu, T K) {
-  const T m0 = a + b + c;
-  const T d = c - a;
-  const T s = c + a;
-  const T m0k = m0 + K;
-  a = m0;
-  b = d - u * m0k;
-  c = s - T(2) * u * d + uu * m0k;
-}
-template <class T>
-__device__ __forceinline__ void inv_line(T& a, T& b, T& c, T u, T uu, T K) {
-  const T m0 = a, m1 = b, m2 = c;
-  const T m0k = m0 + K;
-  const T gm = T(0.5) * ((uu - u) * m0k + (T(2) * u - T(1)) * m1 + m2);
-  const T gp = T(0.5) * ((uu + u) * m0k + (T(2) * u + T(1)) * m1 + m2);
-  const T g0 = m0 * (T(1) - uu) - T(2) * u * m1 - m2 - K * uu;
-  a = gm;
-  b = g0;
-  c = gp;
-}
-
-template <class T>
-__device__ __forceinline__ void to_cube(const T* g, T (&v)[3][3][3]) {
-  static_for<27>([&](auto i) { v[D3Q27::ex(i) + 1][D3Q27::ey(i) + 1][D3Q27::ez(i) + 1] = g[i]; });
-}
-template <class T>
-__device__ __forceinline__ void from_cube(const T (&v)[3][3][3], T* g) {
-  static_for<27>([&](auto i) { g[i] = v[D3Q27::ex(i) + 1][D3Q27::ey(i) + 1][D3Q27::ez(i) + 1]; });
-}
 
 template <class T>
 __device__ __forceinline__ void moments27(const T* g, T& drho, T& jx, T& jy, T& jz) {
