@@ -37,6 +37,7 @@ struct Op {
   enum Kind { GHOSTS, UPDATE, F2C } kind;
   int k = 0;            // finest-level substep of the coarse step the op belongs to
   bool level0 = false;  // level 0 alone, on the graph's branch beside the fine levels (split_level0)
+  bool near = false;    // an update of the level-0 blocks that the fine levels read
   GhostArgs ga{};
   UpdateArgs ua{};
   F2CArgs fa{};
@@ -75,6 +76,7 @@ struct lbm_ctx {
   std::vector<DevLevel> dl;
   WorkItem* items = nullptr;          // merged lists for each lowest level
   std::vector<int64_t> list_off, list_len;
+  int near0 = 0;  // level-0 items (the first of the list) whose blocks level 1 reads or restricts into
   uint32_t* masks = nullptr;
   long long* d_step = nullptr;
   double* partial = nullptr;          // reduction scratch [L][4*sms][4]
@@ -199,11 +201,11 @@ void free_all(lbm_ctx* c) {
 
 // --------------------------------------------------------------- schedule
 // Whether the coarse-step graph runs level 0's work beside the fine levels'
-// chain (nested grids with FP16 storage).  Measured on the paper-scale
-// 3-level jet: FP16 1.454 -> 1.427 ms per coarse step (its half-scale copy
-// 0.303 -> 0.280); FP32 2.100 -> 2.204 ms and the 2-level FP32 jets 1-2 %
-// slower, where the level-0 update is bandwidth-bound on its own and the
-// two branches only compete for DRAM and L2.
+// chain (nested grids with FP16 storage).  Measured, us per coarse step merged
+// -> beside: the paper-scale 3-level jet 1353 -> 1328, its half-scale copy 272
+// -> 250, a small 2-level D3Q19 jet 100.5 -> 98.  FP32 loses (2-level jet 913 ->
+// 1073): its update keeps twice the bytes in flight in the L1, which the shared
+// memory of a coarse-to-fine launch on the same SM takes away.
 bool split_level0(const lbm_ctx* c) { return c->L > 1 && c->storage == LBM_F16; }
 
 std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
@@ -345,15 +347,21 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
     u.step_inc = k == K - 1 && !c->plan.periodic_x ? c->d_step : nullptr;
     up.k = k;
     if (branch0) {
-      // the first substep updates level 0 in a launch of its own: nothing
-      // reads its result before the midpoint of the coarse step, so the
-      // graph runs it beside the fine levels' first half
+      // the first substep updates level 0 in launches of its own: the fine
+      // levels read the blocks near them (the first near0 of the list) from
+      // the midpoint of the coarse step on, and none of the others
+      const int n0 = int(c->list_len[0] - c->list_len[1]);
       Op u0 = up;
       u0.level0 = true;
-      u0.ua.nitems = int(c->list_len[0] - c->list_len[1]);
+      u0.near = true;
+      u0.ua.nitems = c->near0;
+      ops.push_back(u0);
+      u0.near = false;
+      u0.ua.items += c->near0;
+      u0.ua.nitems = n0 - c->near0;
+      if (u0.ua.nitems > 0) ops.push_back(u0);
       up.ua.items = c->items + c->list_off[1];
       up.ua.nitems = int(c->list_len[1]);
-      ops.push_back(u0);
     }
     ops.push_back(up);
     for (int l = lmin; l < L; ++l) par[l] ^= 1;
@@ -380,12 +388,8 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
         v.tau0_c = cp.tau0;
         v.tau0_f = fp.tau0;
         a.n += v.n;
-        op.level0 = l == 1;
       }
       op.k = k;
-      // a restriction into level 0 alone: nothing later in the coarse step
-      // touches level 0, so the graph runs it beside the rest
-      op.level0 = op.level0 && a.nlv == 1 && split_level0(c);
       if (a.n > 0) ops.push_back(op);
     }
   }
@@ -469,16 +473,16 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
       *out = ctx->fork_join[ev++];
       return cudaSuccess;
     };
-    // Nested FP16 grids: the chain of ops runs on the high-priority stream `fine`;
-    // level 0's ghosts and update of the first substep run on the capturing
-    // stream beside it and join the chain before the first op of the second
-    // half of the coarse step (the coarse-to-fine launch that reads level 0's
-    // new state, the restriction into level 0); that restriction in turn runs
-    // beside the rest of the chain (nothing after it touches level 0).  The
-    // level-0 blocks fill the SMs the short interface launches leave idle.
+    // Nested grids: the chain of the fine levels' ops runs on the
+    // high-priority stream `fine`; level 0's ghosts and update run on the
+    // capturing stream beside it.  The chain waits, before the first op of the
+    // second half of the coarse step (the coarse-to-fine launch that reads
+    // level 0's new state, then the restriction into level 0), for the level-0
+    // blocks near the fine levels alone; all others have until the end of the
+    // step and fill the SMs that the short interface launches leave idle.
     const bool split = split_level0(ctx);
     cudaStream_t st = ctx->stream;
-    cudaEvent_t u0_done = nullptr, r0_done = nullptr, evt = nullptr;
+    cudaEvent_t near_done = nullptr, evt = nullptr;
     if (split) {
       if ((e = next_event(&evt)) == cudaSuccess && (e = cudaEventRecord(evt, ctx->stream)) == cudaSuccess)
         e = cudaStreamWaitEvent(ctx->fine, evt, 0);
@@ -487,33 +491,21 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
     const bool chain = chain_launches(ctx);
     for (size_t k = 0; k < ops.size() && e == cudaSuccess; ++k) {
       const Op& op = ops[k];
-      if (u0_done && op.k >= K / 2) {
-        if ((e = cudaStreamWaitEvent(st, u0_done, 0)) != cudaSuccess) break;
-        u0_done = nullptr;
+      if (near_done && op.k >= K / 2) {
+        if ((e = cudaStreamWaitEvent(st, near_done, 0)) != cudaSuccess) break;
+        near_done = nullptr;
       }
-      if (op.level0 && op.kind != Op::F2C) {
+      if (op.level0) {
         if ((e = run_op(ctx, op, ctx->stream)) != cudaSuccess) break;
-        if (op.kind == Op::UPDATE && ((e = next_event(&u0_done)) != cudaSuccess ||
-                                      (e = cudaEventRecord(u0_done, ctx->stream)) != cudaSuccess))
-          break;
-        continue;
-      }
-      if (op.level0 && !u0_done && !r0_done) {
-        // after the chain so far; joined at the end of the coarse step
-        cudaEvent_t here = nullptr;
-        if ((e = next_event(&here)) != cudaSuccess || (e = cudaEventRecord(here, st)) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(ctx->stream, here, 0)) != cudaSuccess ||
-            (e = run_op(ctx, op, ctx->stream)) != cudaSuccess || (e = next_event(&r0_done)) != cudaSuccess ||
-            (e = cudaEventRecord(r0_done, ctx->stream)) != cudaSuccess)
+        if (op.near && ((e = next_event(&near_done)) != cudaSuccess ||
+                        (e = cudaEventRecord(near_done, ctx->stream)) != cudaSuccess))
           break;
         continue;
       }
       if ((e = run_op(ctx, op, st, chain && (s > 0 || k > 0))) != cudaSuccess) break;
     }
     if (split && e == cudaSuccess) {
-      if (u0_done) e = cudaStreamWaitEvent(st, u0_done, 0);
-      if (r0_done && e == cudaSuccess) e = cudaStreamWaitEvent(st, r0_done, 0);
-      if (e == cudaSuccess && (e = next_event(&evt)) == cudaSuccess && (e = cudaEventRecord(evt, st)) == cudaSuccess)
+      if ((e = next_event(&evt)) == cudaSuccess && (e = cudaEventRecord(evt, st)) == cudaSuccess)
         e = cudaStreamWaitEvent(ctx->stream, evt, 0);
     }
   }
@@ -907,9 +899,9 @@ int create_context(lbm_ctx** out, lbm_model model, lbm_storage storage, const lb
     if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ctx->fine, cudaStreamNonBlocking, greatest);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(ce));
   }
-  // events of one coarse step's branches: the fork, level 0 updated, the
-  // restriction's fork and join, the end
-  ctx->fork_join.assign(5, nullptr);
+  // events of one coarse step's branches: the fork, the near blocks updated,
+  // the end
+  ctx->fork_join.assign(3, nullptr);
   for (cudaEvent_t& e : ctx->fork_join) {
     ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("event: ") + cudaGetErrorString(ce));
@@ -951,6 +943,15 @@ int create_context(lbm_ctx** out, lbm_model model, lbm_storage storage, const lb
     }
   }
   if (masks.size() / 16 > 32767) return bail(LBM_ERR_ARG, "too many masked blocks");
+  if (ctx->L > 1) {
+    // level 0's list: first the blocks that level 1's ghosts are interpolated
+    // from or that it restricts into
+    std::vector<char> near(size_t(ctx->plan.lv[0].nblocks()), 0);
+    for (const C2FCell& c : ctx->plan.lv[1].c2f_cells) near[c.cblock] = 1;
+    for (const F2CItem& it : ctx->plan.lv[0].f2c) near[it.cblock] = 1;
+    ctx->near0 = int(std::stable_partition(per[0].begin(), per[0].end(),
+                                           [&](const WorkItem& w) { return near[w.block] != 0; }) - per[0].begin());
+  }
   ctx->list_off.assign(ctx->L, 0);
   ctx->list_len.assign(ctx->L, 0);
   for (int lmin = 0; lmin < ctx->L; ++lmin) {
