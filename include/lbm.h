@@ -13,9 +13,10 @@
  *   - Return value: LBM_OK (0) or a negative lbm_status.  Nothing throws.
  *     lbm_last_error() returns a message for the last failure on a context.
  *   - The context owns all device memory it allocates.  The caller owns every
- *     buffer it passes; host buffers may be pageable or pinned.  The dense
- *     arrays of state, fields, force and gradients may also lie in memory of
- *     the context's device; the caller's own work on them has to be done.
+ *     buffer it passes; host buffers may be pageable or pinned.  The arrays
+ *     of lbm_init_equilibrium, lbm_set_state, lbm_get_state, lbm_macroscopic,
+ *     lbm_set_force and lbm_adjoint_backward may also lie in memory of the
+ *     context's device; the caller's own work on them has to be done.
  *   - Calls are ordered on the context's stream.  lbm_step() only enqueues
  *     work; every call that returns data to the host synchronises the stream.
  *   - Dense per-level arrays are row-major with x fastest: index
@@ -316,7 +317,7 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* dLdf_T, double* dLdF);
 /* Kernel timing: when enabled, lbm_step launches kernels directly (no graph)
  * between CUDA events on the context stream and accumulates per-kind device
  * time.  kinds: 0 update (stream-collide), 1 coarse-to-fine (with the boundary
- * ghosts and nozzle links that share its launch), 2 fine-to-coarse, 3 boundary, 4 other (nothing of a step; an lbm_adjoint_backward call adds the device time of
+ * ghosts and nozzle links of the same substep), 2 fine-to-coarse, 3 boundary, 4 other (nothing of a step; an lbm_adjoint_backward call adds the device time of
  * its recompute + adjoint sweep here as one entry).  ms[k] total
  * milliseconds, launches[k] launch counts. */
 int lbm_set_profiling(lbm_ctx* ctx, int enable);

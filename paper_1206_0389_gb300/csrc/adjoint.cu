@@ -90,12 +90,12 @@ __device__ __forceinline__ void collide27_adjoint(const T* g, T* lam, T om1, T F
   // ---- lines along z
   const T zero = T(0);
   T cz[3], rz[3], xz[3], yz[3], hz[3], qz[3];
-  emit_line<T, false>(drho, Ez * rho, pz, cz[0], cz[1], cz[2]);
-  emit_line<T, false>(zero, uz * kyz, kyz, rz[0], rz[1], rz[2]);
-  emit_line<T, false>(zero, uz * kxz, kxz, xz[0], xz[1], xz[2]);
-  emit_line<T, false>(kxy, Ez * kxy, uz * kxy, yz[0], yz[1], yz[2]);
-  emit_line<T, false>(T(1), T(0.5) * uz * uz - T(1.0 / 6.0), uz, hz[0], hz[1], hz[2]);
-  emit_line<T, false>(zero, uz * fz, fz, qz[0], qz[1], qz[2]);
+  emit_line<T>(drho, Ez * rho, pz, cz[0], cz[1], cz[2]);
+  emit_line<T>(zero, uz * kyz, kyz, rz[0], rz[1], rz[2]);
+  emit_line<T>(zero, uz * kxz, kxz, xz[0], xz[1], xz[2]);
+  emit_line<T>(kxy, Ez * kxy, uz * kxy, yz[0], yz[1], yz[2]);
+  emit_line<T>(T(1), T(0.5) * uz * uz - T(1.0 / 6.0), uz, hz[0], hz[1], hz[2]);
+  emit_line<T>(zero, uz * fz, fz, qz[0], qz[1], qz[2]);
   // ---- per z layer: lines along y again, then the x and y lines reversed;
   // the adjoint of each z value takes its place
   T Exb = zero, Eyb = zero, Ezb = zero, Hxb = zero, Hyb = zero;
@@ -104,9 +104,9 @@ __device__ __forceinline__ void collide27_adjoint(const T* g, T* lam, T om1, T F
   for (int k = 0; k < 3; ++k) {
     const T A = cz[k] + T(w1(k)), f = fx * hz[k], q = fy * hz[k];
     T cy[3], ry[3], gy[3];
-    emit_line<T, false>(cz[k], Ey * A + uy * rz[k], uy * A + rz[k], cy[0], cy[1], cy[2]);
-    emit_line<T, false>(xz[k] + f, Ey * xz[k] + uy * yz[k] + Hy * f, uy * (xz[k] + f) + yz[k], ry[0], ry[1], ry[2]);
-    emit_line<T, false>(qz[k], Hy * qz[k] + uy * q, uy * qz[k] + q, gy[0], gy[1], gy[2]);
+    emit_line<T>(cz[k], Ey * A + uy * rz[k], uy * A + rz[k], cy[0], cy[1], cy[2]);
+    emit_line<T>(xz[k] + f, Ey * xz[k] + uy * yz[k] + Hy * f, uy * (xz[k] + f) + yz[k], ry[0], ry[1], ry[2]);
+    emit_line<T>(qz[k], Hy * qz[k] + uy * q, uy * qz[k] + q, gy[0], gy[1], gy[2]);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const LineAdj<T> l(lam[D3Q27::index(-1, b - 1, k - 1)], lam[D3Q27::index(0, b - 1, k - 1)],

@@ -67,9 +67,10 @@ struct lbm_ctx {
   double omega = 1.0, cs = 0.0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  // stream and events of the coarse-step graph's branches: the fine-level
-  // chain (fine, high priority) beside the level-0 update (the capturing stream)
-  cudaStream_t fine = nullptr;
+  // streams and events of the coarse-step graph's branches: the inflow
+  // launch beside the coarse-to-fine launch (side), and the fine-level chain
+  // (fine, high priority) beside the level-0 update (the capturing stream)
+  cudaStream_t side = nullptr, fine = nullptr;
   std::vector<cudaEvent_t> fork_join;
   int device = 0, sms = 1;
   bool host_direct = false;  // kernels reach ordinary host memory through the host's page tables
@@ -195,6 +196,7 @@ void free_all(lbm_ctx* c) {
   cudaFree(c->stage);
   release_adjoint(c);
   for (cudaEvent_t e : c->fork_join) cudaEventDestroy(e);
+  if (c->side) cudaStreamDestroy(c->side);
   if (c->fine) cudaStreamDestroy(c->fine);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
@@ -224,9 +226,8 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
         break;
       }
     auto sub = [&](int l) { return k / (1 << (L - 1 - l)); };
-    // one launch for all that the levels starting a substep pull from outside
-    // their updated cells; where level 0 has a branch of its own, its part
-    // goes there
+    // all that the levels starting a substep pull from outside their updated
+    // cells; where level 0 has a branch of its own, its part goes there
     auto ghosts = [&](int l_lo, int l_hi, bool level0) {
       Op op;
       op.kind = Op::GHOSTS;
@@ -407,7 +408,7 @@ bool chain_launches(const lbm_ctx* c) { return c->L == 1 && c->storage != LBM_F6
 
 cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st, bool chained = false) {
   switch (op.kind) {
-    case Op::GHOSTS: return launch_ghosts(c->model, c->storage, op.ga, chained, st);
+    case Op::GHOSTS: return launch_ghosts(c->model, c->storage, op.ga, st);
     case Op::UPDATE: {
       UpdateArgs a = op.ua;
       a.chained = chained;
@@ -418,8 +419,7 @@ cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st, bool chained = fal
   return cudaErrorInvalidValue;
 }
 
-// kinds of lbm_get_profile (a launch of several kinds of ghosts counts as
-// coarse-to-fine)
+// kinds of lbm_get_profile (ghosts of several kinds count as coarse-to-fine)
 int op_kind_index(const Op& op) {
   switch (op.kind) {
     case Op::GHOSTS: return op.ga.c2f.n > 0 ? 1 : 3;
@@ -499,6 +499,22 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
         if ((e = run_op(ctx, op, ctx->stream)) != cudaSuccess) break;
         if (op.near && ((e = next_event(&near_done)) != cudaSuccess ||
                         (e = cudaEventRecord(near_done, ctx->stream)) != cudaSuccess))
+          break;
+        continue;
+      }
+      if (op.kind == Op::GHOSTS && op.ga.c2f.n > 0 && op.ga.bc.n > 0) {
+        // the inflow launch touches other cells than the coarse-to-fine launch
+        // (which writes the inflow ghosts fed by its own), so the two run side
+        // by side
+        cudaEvent_t fork = nullptr, join = nullptr;
+        if ((e = next_event(&fork)) != cudaSuccess || (e = next_event(&join)) != cudaSuccess ||
+            (e = cudaEventRecord(fork, st)) != cudaSuccess ||
+            (e = cudaStreamWaitEvent(ctx->side, fork, 0)) != cudaSuccess ||
+            (e = launch_bc(ctx->model, ctx->storage, op.ga.bc, ctx->side)) != cudaSuccess ||
+            (e = launch_c2f(ctx->model, ctx->storage, op.ga.c2f, st)) != cudaSuccess ||
+            (e = launch_links(ctx->model, ctx->storage, op.ga.link, st)) != cudaSuccess ||
+            (e = cudaEventRecord(join, ctx->side)) != cudaSuccess ||
+            (e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess)
           break;
         continue;
       }
@@ -896,12 +912,13 @@ int create_context(lbm_ctx** out, lbm_model model, lbm_storage storage, const lb
     // stream priority, the level-0 update beside it at the caller's
     int least = 0, greatest = 0;
     ce = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest);
     if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&ctx->fine, cudaStreamNonBlocking, greatest);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(ce));
   }
   // events of one coarse step's branches: the fork, the near blocks updated,
-  // the end
-  ctx->fork_join.assign(3, nullptr);
+  // the end, and a fork and a join per coarse-to-fine launch
+  ctx->fork_join.assign(3 + 2 * (1 << (ctx->L - 1)), nullptr);
   for (cudaEvent_t& e : ctx->fork_join) {
     ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("event: ") + cudaGetErrorString(ce));

@@ -198,6 +198,60 @@ __device__ __forceinline__ T collide19(T* g, T tau0, T cs2_18) {
   return T(1.5) * Qn / tau;
 }
 
+// The same collision in float64, whose pipes bound the update: the sums of the
+// two pairs of each plane serve all moments (48 additions instead of 63), the
+// squares of u serve every link, and one reciprocal of tau_total serves k and
+// |S|.  32^3 D3Q19 FP64: F64_19 us per step.
+__device__ __forceinline__ double collide19_f64(double* g, double tau0, double cs2_18) {
+  double s[9], d[9];
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    s[p] = g[2 * p + 1] + g[2 * p + 2];
+    d[p] = g[2 * p + 1] - g[2 * p + 2];
+  }
+  // pairs 0..2: x, y, z; (3, 4), (5, 6), (7, 8): the diagonals of xy, xz, yz
+  const double Exy = s[3] + s[4], Exz = s[5] + s[6], Eyz = s[7] + s[8];
+  const double sxy = s[3] - s[4], sxz = s[5] - s[6], syz = s[7] - s[8];
+  const double ux = d[0] + (d[3] + d[4]) + (d[5] + d[6]);
+  const double uy = d[1] + (d[3] - d[4]) + (d[7] + d[8]);
+  const double uz = d[2] + (d[5] - d[6]) + (d[7] - d[8]);
+  const double drho = g[0] + ((s[0] + s[1]) + s[2]) + ((Exy + Exz) + Eyz);
+  const double xx = ux * ux, yy = uy * uy, zz = uz * uz, d3 = drho * (1.0 / 3.0);
+  const double pxx = s[0] + Exy + Exz - d3 - xx, pyy = s[1] + Exy + Eyz - d3 - yy, pzz = s[2] + Exz + Eyz - d3 - zz;
+  const double pxy = sxy - ux * uy, pxz = sxz - ux * uz, pyz = syz - uy * uz;
+  const double qq = 2.0 * (pxx * pxx + pyy * pyy + pzz * pzz) + 4.0 * (pxy * pxy + pxz * pxz + pyz * pyz);
+  const double Qn = sqrt(qq);
+  const double inv = 2.0 / (tau0 + sqrt(tau0 * tau0 + cs2_18 * Qn));  // 1 / tau_total
+  const double k = 1.0 - inv, k2 = 0.5 * k, k4 = 0.25 * k;
+  const double tr3 = (pxx + pyy + pzz) * (1.0 / 3.0);
+  const double base = drho - 1.5 * (xx + yy + zz);
+  g[0] = (1.0 / 3.0) * base;
+  const double b1 = (1.0 / 18.0) * base, b2 = (1.0 / 36.0) * base;
+  // axis links: w (base + 4.5 u_a^2) + k/2 (Pi_aa - tr Pi / 3) +- u_a / 6
+  auto axis = [&](int i, double u, double uu, double pi) {
+    const double sym = b1 + 0.25 * uu + k2 * (pi - tr3), asym = (1.0 / 6.0) * u;
+    g[i] = sym + asym;
+    g[i + 1] = sym - asym;
+  };
+  axis(1, ux, xx, pxx);
+  axis(3, uy, yy, pyy);
+  axis(5, uz, zz, pzz);
+  // diagonals: w (base + 4.5 (u_a +- u_b)^2) +- k/4 Pi_ab +- (u_a +- u_b) / 12
+  const double hx = (1.0 / 12.0) * ux, hy = (1.0 / 12.0) * uy, hz = (1.0 / 12.0) * uz;
+  auto plane = [&](int i, double ua, double ub, double aa, double bb, double ha, double hb, double pi) {
+    const double even = b2 + 0.125 * (aa + bb), odd = 0.25 * ua * ub + k4 * pi;
+    const double sp = even + odd, sm = even - odd, ap = ha + hb, am = ha - hb;
+    g[i] = sp + ap;
+    g[i + 1] = sp - ap;
+    g[i + 2] = sm + am;
+    g[i + 3] = sm - am;
+  };
+  plane(7, ux, uy, xx, yy, hx, hy, pxy);
+  plane(11, ux, uz, xx, zz, hx, hz, pxz);
+  plane(15, uy, uz, yy, zz, hy, hz, pyz);
+  return 1.5 * Qn * inv;
+}
+
 // ------------------------------------------------------------------ D3Q27 FCLB
 // one-dimensional weights (index 0/1/2 means velocity -1/0/+1)
 __host__ __device__ constexpr double w1(int k) { return k == 1 ? 2.0 / 3.0 : 1.0 / 6.0; }
@@ -220,7 +274,7 @@ __device__ __forceinline__ void moments27(const T* g, T& drho, T& jx, T& jy, T& 
 // fourth M_aa M_bb and M_aa M_bc, sixth M11 M22 M33).  With a body force F,
 // u = (j + F/2)/rho and the first central moments leave as F/(2 rho).
 //
-// In closed form, used by the stream-collide kernel with FP32 storage.
+// In closed form, used by the stream-collide kernels with FP32 and FP16 storage.
 // Because every moment above second order is relaxed with rate 1, only the
 // six pre-collision second-order central moments matter; they follow from
 // raw sums: rho kappa_aa = S_aa - 2 u_a j_a + u_a^2 rho (+ const), rho kappa_ab =
@@ -234,7 +288,10 @@ __device__ __forceinline__ void moments27(const T* g, T& drho, T& jx, T& jy, T& 
 // keeps f* - w free of cancellation:
 //   f*_i - w_i = drho W_i + rho (dx Py Pz... expanded) + k_xy psi_x psi_y phi_z + ...
 // (the paper notes that fixed rates remove most of the FCLB flops).
-template <class T, bool Force>
+// Scaled: g holds g_i / w_i on entry and exit (the FP16 storage form); the
+// product weights w_i = w1_x w1_y w1_z then enter once per z-line on input
+// and once per (e_y, e_z) pair and per e_x factor on output.
+template <class T, bool Force, bool Scaled = false>
 __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz) {
   // ---- zeroth, first and second raw moments of g by a z, y, x collapse
   T m0[3][3], dz[3][3], sz[3][3];  // per (ex, ey): sum, difference, sum of ends along z
@@ -245,9 +302,16 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
       const T lo = g[D3Q27::index(a - 1, b - 1, -1)];
       const T mi = g[D3Q27::index(a - 1, b - 1, 0)];
       const T hi = g[D3Q27::index(a - 1, b - 1, 1)];
-      sz[a][b] = hi + lo;
-      dz[a][b] = hi - lo;
-      m0[a][b] = sz[a][b] + mi;
+      if constexpr (Scaled) {
+        const T ce = T(w1(a) * w1(b) * w1(0)), cm = T(w1(a) * w1(b) * w1(1));
+        sz[a][b] = ce * (hi + lo);
+        dz[a][b] = ce * (hi - lo);
+        m0[a][b] = sz[a][b] + cm * mi;
+      } else {
+        sz[a][b] = hi + lo;
+        dz[a][b] = hi - lo;
+        m0[a][b] = sz[a][b] + mi;
+      }
     }
   T M0[3], My[3], Myy[3], Dz[3], Dyz[3], Szz[3];
 #pragma unroll
@@ -315,20 +379,47 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
     }
   }
   // ---- per (e_y, e_z) pair, then per e_x
+  if constexpr (Scaled) {
+    // the x factors divided by w1_x once
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      dl[0][a] *= T(1.0 / w1(a));
+      ps[0][a] *= T(1.0 / w1(a));
+      ph[0][a] *= T(1.0 / w1(a));
+      if constexpr (Force) ch[0][a] *= T(1.0 / w1(a));
+    }
+  }
 #pragma unroll
   for (int b = 0; b < 3; ++b)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const T P = ph[1][b] * ph[2][c];                            // phi_y phi_z
       const T Qd = T(w1(b)) * dl[2][c] + dl[1][b] * ph[2][c];     // phi_y phi_z - w1_y w1_z
-      const T rP = rho * P, rQ = rho * Qd;
-      const T R = kxy * ps[1][b] * ph[2][c] + kxz * ph[1][b] * ps[2][c];
-      const T Sy = kyz * ps[1][b] * ps[2][c];
+      T rP = rho * P, rQ = rho * Qd;
+      T R = kxy * ps[1][b] * ph[2][c] + kxz * ph[1][b] * ps[2][c];
+      T Sy = kyz * ps[1][b] * ps[2][c];
       T Fp = T(0), Gp = T(0);
       if constexpr (Force) {
         Fp = T(0.5) * Fx * ch[1][b] * ch[2][c];
         Gp = T(0.5) * Fy * ps[1][b] * ch[2][c] + T(0.5) * Fz * ch[1][b] * ps[2][c];
       }
+      if constexpr (Scaled) {
+        const T ibc = T(1.0 / (w1(b) * w1(c)));
+        rP *= ibc;
+        R *= ibc;
+        Sy *= ibc;
+        if constexpr (Force) {
+          Fp *= ibc;
+          Gp *= ibc;
+        }
+        const T base = drho + ibc * rQ;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          T v = base + dl[0][a] * rP + ps[0][a] * R + ph[0][a] * Sy;
+          if constexpr (Force) v += ps[0][a] * Fp + ch[0][a] * Gp;
+          g[D3Q27::index(a - 1, b - 1, c - 1)] = v;
+        }
+      } else {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           const T W = T(w1(a) * w1(b) * w1(c));
@@ -336,11 +427,12 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
           if constexpr (Force) v += ps[0][a] * Fp + ch[0][a] * Gp;
           g[D3Q27::index(a - 1, b - 1, c - 1)] = v;
         }
+      }
     }
 }
 
 // The collision of collide27_closed as nested one-dimensional lines, for FP64
-// and FP16 storage.  A line is the three values along one axis of
+// storage.  A line is the three values along one axis of
 //   c w1(e) + A delta(e) + R psi(e),   delta(+-1) = E +- u/2, delta(0) = -2 E,
 //   psi(+-1) = u +- 1/2, psi(0) = -2 u,  E = (u^2 + D) / 2,
 // which come in pairs: with t = E A + u R the even part is c/6 + t, the odd
@@ -349,34 +441,20 @@ __device__ __forceinline__ void collide27_closed(T* g, T omega, T Fx, T Fy, T Fz
 // value c found gives the next axis its A = c + w, and kyz psi_z its R; the
 // shear terms kxy phi_z, kxz psi_z make a second line along y that is the R of
 // the x lines.  About 245 operations a cell against 400 of collide27_closed,
-// and fewer values alive (112 registers against 212 in float64 without a cap):
-// 128^3 FP64, bound by the float64 pipes, 1313 -> 1006 us per step; 256^3 FP16
-// 300 -> 287 us.  The last bits differ, so FP32 storage, bound by memory,
-// keeps that form.
-// Scaled (FP16 storage): values are g_i / w_i; all sums run in units of
-// products of 1/6 (a middle value weighs 4, exactly) and lines have no weights.
-// om1 = 1 - omega.
-template <class T, bool Scaled>
+// and fewer values alive (112 registers against 212 without a cap): 128^3, bound
+// by the float64 pipes, 1313 -> 1006 us per step.  The last bits differ, which
+// FP32 and FP16 runs show as drifts and flipped roundings of the storage, so
+// those, bound by memory, keep the other form.  om1 = 1 - omega.
+template <class T>
 __device__ __forceinline__ void emit_line(T c, T t, T odd, T& lo, T& mid, T& hi) {
-  if constexpr (Scaled) {
-    mid = c - T(3) * t;
-    const T ev = c + T(6) * t;
-    lo = ev - T(3) * odd;
-    hi = ev + T(3) * odd;
-  } else {
-    const T ev = T(1.0 / 6.0) * c + t;
-    mid = c - T(2) * ev;
-    lo = ev - T(0.5) * odd;
-    hi = ev + T(0.5) * odd;
-  }
+  const T ev = T(1.0 / 6.0) * c + t;
+  mid = c - T(2) * ev;
+  lo = ev - T(0.5) * odd;
+  hi = ev + T(0.5) * odd;
 }
-template <class T, bool Force, bool Scaled>
+template <class T, bool Force>
 __device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
   // ---- raw moments up to second order by a z, y, x collapse
-  auto centre = [](T ends, T mid) -> T {
-    if constexpr (Scaled) return T(4) * mid + ends;
-    else return ends + mid;
-  };
   T m0[3][3], dz[3][3], sz[3][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -385,38 +463,25 @@ __device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
       const T lo = g[D3Q27::index(a - 1, b - 1, -1)], hi = g[D3Q27::index(a - 1, b - 1, 1)];
       sz[a][b] = hi + lo;
       dz[a][b] = hi - lo;
-      m0[a][b] = centre(sz[a][b], g[D3Q27::index(a - 1, b - 1, 0)]);
+      m0[a][b] = (sz[a][b]) + g[D3Q27::index(a - 1, b - 1, 0)];
     }
   T M0[3], My[3], Myy[3], Dz[3], Dyz[3], Szz[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     Myy[a] = m0[a][2] + m0[a][0];
     My[a] = m0[a][2] - m0[a][0];
-    M0[a] = centre(Myy[a], m0[a][1]);
-    Dz[a] = centre(dz[a][2] + dz[a][0], dz[a][1]);
+    M0[a] = (Myy[a]) + m0[a][1];
+    Dz[a] = (dz[a][2] + dz[a][0]) + dz[a][1];
     Dyz[a] = dz[a][2] - dz[a][0];
-    Szz[a] = centre(sz[a][2] + sz[a][0], sz[a][1]);
+    Szz[a] = (sz[a][2] + sz[a][0]) + sz[a][1];
   }
   T Sxx = M0[2] + M0[0], jx = M0[2] - M0[0];
-  T drho = centre(Sxx, M0[1]);
-  T jy = centre(My[2] + My[0], My[1]), Sxy = My[2] - My[0];
-  T Syy = centre(Myy[2] + Myy[0], Myy[1]);
-  T jz = centre(Dz[2] + Dz[0], Dz[1]), Sxz = Dz[2] - Dz[0];
-  T Syz = centre(Dyz[2] + Dyz[0], Dyz[1]);
-  T Szzt = centre(Szz[2] + Szz[0], Szz[1]);
-  if constexpr (Scaled) {
-    const T w = T(1.0 / 216.0);
-    Sxx = Sxx * w;
-    Syy = Syy * w;
-    Szzt = Szzt * w;
-    Sxy = Sxy * w;
-    Sxz = Sxz * w;
-    Syz = Syz * w;
-    drho = drho * w;
-    jx = jx * w;
-    jy = jy * w;
-    jz = jz * w;
-  }
+  T drho = (Sxx) + M0[1];
+  T jy = (My[2] + My[0]) + My[1], Sxy = My[2] - My[0];
+  T Syy = (Myy[2] + Myy[0]) + Myy[1];
+  T jz = (Dz[2] + Dz[0]) + Dz[1], Sxz = Dz[2] - Dz[0];
+  T Syz = (Dyz[2] + Dyz[0]) + Dyz[1];
+  T Szzt = (Szz[2] + Szz[0]) + Szz[1];
   // ---- velocity, second-order central moments, relaxation
   const T rho = T(1) + drho;
   const T r = T(1) / rho;
@@ -452,49 +517,49 @@ __device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
   // ---- lines along z: rho phi_z - w, kyz psi_z, kxz psi_z, kxy phi_z
   const T zero = T(0);
   T cz[3], rz[3], xz[3], yz[3];
-  emit_line<T, Scaled>(drho, Ez * rho, pz, cz[0], cz[1], cz[2]);
-  emit_line<T, Scaled>(zero, uz * kyz, kyz, rz[0], rz[1], rz[2]);
-  emit_line<T, Scaled>(zero, uz * kxz, kxz, xz[0], xz[1], xz[2]);
-  emit_line<T, Scaled>(kxy, Ez * kxy, uz * kxy, yz[0], yz[1], yz[2]);
+  emit_line<T>(drho, Ez * rho, pz, cz[0], cz[1], cz[2]);
+  emit_line<T>(zero, uz * kyz, kyz, rz[0], rz[1], rz[2]);
+  emit_line<T>(zero, uz * kxz, kxz, xz[0], xz[1], xz[2]);
+  emit_line<T>(kxy, Ez * kxy, uz * kxy, yz[0], yz[1], yz[2]);
   // the force's first-order moments have no second-order part: chi = (1, 0, 0)
   T hz[3], qz[3], Hx = zero, Hy = zero, Hz = zero;
   if constexpr (Force) {
     Hx = T(0.5) * ux * ux - T(1.0 / 6.0);
     Hy = T(0.5) * uy * uy - T(1.0 / 6.0);
     Hz = T(0.5) * uz * uz - T(1.0 / 6.0);
-    emit_line<T, Scaled>(T(1), Hz, uz, hz[0], hz[1], hz[2]);
+    emit_line<T>(T(1), Hz, uz, hz[0], hz[1], hz[2]);
     const T f = T(0.5) * Fz;
-    emit_line<T, Scaled>(zero, uz * f, f, qz[0], qz[1], qz[2]);
+    emit_line<T>(zero, uz * f, f, qz[0], qz[1], qz[2]);
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     // ---- lines along y at this e_z
-    const T A = cz[k] + T(Scaled ? 1.0 : w1(k));
+    const T A = cz[k] + T(w1(k));
     T cy[3], ry[3], gy[3];
-    emit_line<T, Scaled>(cz[k], Ey * A + uy * rz[k], uy * A + rz[k], cy[0], cy[1], cy[2]);
-    emit_line<T, Scaled>(xz[k], Ey * xz[k] + uy * yz[k], uy * xz[k] + yz[k], ry[0], ry[1], ry[2]);
+    emit_line<T>(cz[k], Ey * A + uy * rz[k], uy * A + rz[k], cy[0], cy[1], cy[2]);
+    emit_line<T>(xz[k], Ey * xz[k] + uy * yz[k], uy * xz[k] + yz[k], ry[0], ry[1], ry[2]);
     if constexpr (Force) {
       // Fx/2 chi_y chi_z joins the x lines' R; Fy/2 psi_y chi_z + Fz/2 chi_y psi_z
       // is their chi slot
       const T f = T(0.5) * Fx * hz[k], q = T(0.5) * Fy * hz[k];
       T lo, mid, hi;
-      emit_line<T, Scaled>(f, Hy * f, uy * f, lo, mid, hi);
+      emit_line<T>(f, Hy * f, uy * f, lo, mid, hi);
       ry[0] += lo;
       ry[1] += mid;
       ry[2] += hi;
-      emit_line<T, Scaled>(qz[k], Hy * qz[k] + uy * q, uy * qz[k] + q, gy[0], gy[1], gy[2]);
+      emit_line<T>(qz[k], Hy * qz[k] + uy * q, uy * qz[k] + q, gy[0], gy[1], gy[2]);
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       // ---- lines along x
-      const T Ax = cy[b] + T(Scaled ? 1.0 : w1(b) * w1(k));
+      const T Ax = cy[b] + T(w1(b) * w1(k));
       T& lo = g[D3Q27::index(-1, b - 1, k - 1)];
       T& mid = g[D3Q27::index(0, b - 1, k - 1)];
       T& hi = g[D3Q27::index(1, b - 1, k - 1)];
       if constexpr (Force)
-        emit_line<T, Scaled>(cy[b] + gy[b], Ex * Ax + ux * ry[b] + Hx * gy[b], ux * (Ax + gy[b]) + ry[b], lo, mid, hi);
+        emit_line<T>(cy[b] + gy[b], Ex * Ax + ux * ry[b] + Hx * gy[b], ux * (Ax + gy[b]) + ry[b], lo, mid, hi);
       else
-        emit_line<T, Scaled>(cy[b], Ex * Ax + ux * ry[b], ux * Ax + ry[b], lo, mid, hi);
+        emit_line<T>(cy[b], Ex * Ax + ux * ry[b], ux * Ax + ry[b], lo, mid, hi);
     }
   }
 }
@@ -502,8 +567,8 @@ __device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
 // the form that a storage's update uses
 template <class T, bool Force, bool Scaled>
 __device__ __forceinline__ void collide27(T* g, T omega, T Fx, T Fy, T Fz) {
-  if constexpr (Scaled || std::is_same<T, double>::value) collide27_lines<T, Force, Scaled>(g, T(1) - omega, Fx, Fy, Fz);
-  else collide27_closed<T, Force>(g, omega, Fx, Fy, Fz);
+  if constexpr (std::is_same<T, double>::value) collide27_lines<T, Force>(g, T(1) - omega, Fx, Fy, Fz);
+  else collide27_closed<T, Force, Scaled>(g, omega, Fx, Fy, Fz);
 }
 
 // Product-form D3Q27 equilibrium minus the weights: the distribution whose

@@ -20,7 +20,6 @@
 #include <type_traits>
 
 #include "collide.cuh"
-#include "chained.cuh"
 #include "kernels.cuh"
 
 namespace lbm {
@@ -114,16 +113,6 @@ __device__ __forceinline__ double inflow_u(const long long* step, double y0, dou
                                            double u_in, double perturb, unsigned long long seed,
                                            int level, int substep, int NY, double inv_scale, int y,
                                            int z, int c) {
-  // most face cells lie clearly outside the disc: decided in float32 with a
-  // margin above its rounding (coordinates and their differences are off by
-  // less than 2^-22 of the coordinates' sum, so squares by less than 2^-20 of
-  // its square), which saves the scarce float64 issue slots
-  {
-    const float yf = (float(y) + 0.5f) * float(inv_scale), zf = (float(z) + 0.5f) * float(inv_scale);
-    const float y0f = float(y0), z0f = float(z0), ey = yf - y0f, ez = zf - z0f;
-    const float sy = yf + fabsf(y0f), sz = zf + fabsf(z0f);
-    if (ey * ey + ez * ez - 4e-6f * (sy * sy + sz * sz) > float(r2) * 1.000001f) return 0.0;
-  }
   const double yc = (double(y) + 0.5) * inv_scale;
   const double zc = (double(z) + 0.5) * inv_scale;
   const double dy = yc - y0, dz = zc - z0;
@@ -162,7 +151,7 @@ __device__ __forceinline__ T quad_sum(T v) {
 // per ghost cell interpolates from shared memory.  The distinct cells of a
 // chunk number about a quarter of its 8 x items stencil references.
 template <class M, class S>
-__device__ __forceinline__ void coarse_to_fine(const C2FArgs& a, int chunk) {
+__global__ void __launch_bounds__(kC2FMaxItems) k_c2f(const C2FArgs a) {
   using St = Store<S>;
   using T = typename St::T;
   constexpr int Q = M::Q;
@@ -176,7 +165,7 @@ __device__ __forceinline__ void coarse_to_fine(const C2FArgs& a, int chunk) {
   using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
   __shared__ __align__(16) T sv[MC * QP];
   __shared__ T sS[MC];
-  int g = chunk;
+  int g = blockIdx.x;
   const C2FLevel L = pick_level<C2FLevel>(a, g);
   const C2FChunk ch = L.chunks[g];
   const int nc = ch.ncells;
@@ -341,15 +330,14 @@ __global__ void __launch_bounds__(128) k_f2c(const F2CArgs a) {
 // out), the density is a sum over the eight lanes, and each lane writes its
 // populations with e_x = +1.
 constexpr int kBCLanes = 8;
-constexpr int kGhostTPB = kC2FMaxItems;  // threads per CTA of the launch they share
 
 template <class M, class S>
-__device__ __forceinline__ void boundary(const BCArgs& a, int cta) {
+__global__ void __launch_bounds__(128) k_bc(const BCArgs a) {
   using St = Store<S>;
   using T = typename St::T;
   constexpr int Q = M::Q;
   constexpr int QS = Q * kCells;
-  const int t = cta * kGhostTPB + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int r = t & (kBCLanes - 1);
   const bool valid = (t / kBCLanes) < a.n;
   int n = valid ? t / kBCLanes : a.n - 1;  // tail lanes mirror the last cell
@@ -426,11 +414,11 @@ __device__ __forceinline__ void boundary(const BCArgs& a, int cta) {
 // the shifted storage values unchanged.  On the downstream cap: the inflow
 // equilibrium with the density of the fluid cell straight downstream.
 template <class M, class S>
-__device__ __forceinline__ void nozzle_links(const LinkArgs& a, int cta) {
+__global__ void __launch_bounds__(128) k_links(const LinkArgs a) {
   using T = typename Store<S>::T;
   constexpr int Q = M::Q;
   constexpr int QS = Q * kCells;
-  const int t = cta * kGhostTPB + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.n) return;
   const LinkItem it = a.items[t];
   S* f = reinterpret_cast<S*>(a.f);
@@ -463,44 +451,30 @@ __device__ __forceinline__ void nozzle_links(const LinkArgs& a, int cta) {
   store_rt<S, Q>(f + int64_t(it.bblock) * QS + ib * kCells + it.bcell, ib, v);
 }
 
-// Every value that the levels' next pulls take from outside their updated
-// cells, in one launch: coarse-to-fine chunks (one CTA each, first, as they
-// take longest), inflow and outlet ghosts (16 per CTA), nozzle links (128 per
-// CTA).  The three write different cells and read none of each other's, and
-// each alone is a few microseconds of latency on part of the SMs.  As launches
-// of their own (the inflow beside, the links after the coarse-to-fine launch)
-// -> together, us per coarse step: the small D3Q19 jet 153 -> 146, the small
-// tank 213 -> 203, the full-size 2-level jet 913 -> 911, the paper-scale FP16
-// jet 1329 -> 1333.  Registers are capped where shared memory stops anyway, 7
-// CTAs per SM (D3Q27 6: the next cap spills, which is far slower).
-template <class M, class S, bool C2F>
-__global__ void __launch_bounds__(kGhostTPB, C2F && !std::is_same<S, double>::value ? (M::Q == 19 ? 7 : 6) : 1) k_ghosts(const GhostArgs a) {
-  begin_chained();
-  int cta = blockIdx.x;
-  if constexpr (C2F) {
-    if (cta < a.c2f.n) {
-      coarse_to_fine<M, S>(a.c2f, cta);
-      return;
-    }
-    cta -= a.c2f.n;
-  }
-  const int nb = (a.bc.n + kGhostTPB / kBCLanes - 1) / (kGhostTPB / kBCLanes);
-  if (cta < nb) boundary<M, S>(a.bc, cta);
-  else nozzle_links<M, S>(a.link, cta - nb);
-}
-
+// coarse-to-fine: one CTA per chunk; fine-to-coarse: four lanes per item, 32
+// items per CTA; inflow: eight lanes per item, 16 items per CTA
 template <class M, class S>
-static cudaError_t ghosts_ms(const GhostArgs& a, bool chained, cudaStream_t st) {
-  const int n = a.c2f.n + (a.bc.n + kGhostTPB / kBCLanes - 1) / (kGhostTPB / kBCLanes) + (a.link.n + kGhostTPB - 1) / kGhostTPB;
-  if (n == 0) return cudaSuccess;
-  return a.c2f.n > 0 ? launch_chained(k_ghosts<M, S, true>, n, kGhostTPB, a, chained, st)
-                     : launch_chained(k_ghosts<M, S, false>, n, kGhostTPB, a, chained, st);
+static cudaError_t c2f_ms(const C2FArgs& a, cudaStream_t st) {
+  if (a.n == 0) return cudaSuccess;
+  k_c2f<M, S><<<a.n, kC2FMaxItems, 0, st>>>(a);
+  return cudaGetLastError();
 }
-// fine-to-coarse: four lanes per item, 32 items per CTA
 template <class M, class S>
 static cudaError_t f2c_ms(const F2CArgs& a, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
   k_f2c<M, S><<<(a.n + 31) / 32, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+template <class M, class S>
+static cudaError_t links_ms(const LinkArgs& a, cudaStream_t st) {
+  if (a.n == 0) return cudaSuccess;
+  k_links<M, S><<<(a.n + 127) / 128, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+template <class M, class S>
+static cudaError_t bc_ms(const BCArgs& a, cudaStream_t st) {
+  if (a.n == 0) return cudaSuccess;
+  k_bc<M, S><<<(a.n + 128 / kBCLanes - 1) / (128 / kBCLanes), 128, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -514,9 +488,16 @@ static cudaError_t f2c_ms(const F2CArgs& a, cudaStream_t st) {
   if (storage == LBM_F32) return FN<Fclb, float>(__VA_ARGS__);             \
   return FN<Fclb, __half>(__VA_ARGS__);
 
-cudaError_t launch_ghosts(int model, int storage, const GhostArgs& a, bool chained, cudaStream_t st) {
-  LBM_DISPATCH(ghosts_ms, a, chained, st)
-}
+cudaError_t launch_c2f(int model, int storage, const C2FArgs& a, cudaStream_t st) { LBM_DISPATCH(c2f_ms, a, st) }
 cudaError_t launch_f2c(int model, int storage, const F2CArgs& a, cudaStream_t st) { LBM_DISPATCH(f2c_ms, a, st) }
+cudaError_t launch_bc(int model, int storage, const BCArgs& a, cudaStream_t st) { LBM_DISPATCH(bc_ms, a, st) }
+cudaError_t launch_links(int model, int storage, const LinkArgs& a, cudaStream_t st) { LBM_DISPATCH(links_ms, a, st) }
+
+cudaError_t launch_ghosts(int model, int storage, const GhostArgs& a, cudaStream_t st) {
+  cudaError_t e = launch_c2f(model, storage, a.c2f, st);
+  if (e == cudaSuccess) e = launch_bc(model, storage, a.bc, st);
+  if (e == cudaSuccess) e = launch_links(model, storage, a.link, st);
+  return e;
+}
 
 }  // namespace lbm

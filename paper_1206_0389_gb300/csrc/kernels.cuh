@@ -223,7 +223,7 @@ struct LinkArgs {
   unsigned long long seed;
 };
 
-// what one launch brings in before an update (parts with n = 0 are absent)
+// what is brought in before an update (parts with n = 0 are absent)
 struct GhostArgs {
   C2FArgs c2f;
   BCArgs bc;
@@ -235,7 +235,10 @@ struct GhostArgs {
 cudaError_t launch_update(int model, int storage, const UpdateArgs& a, int threads, int minb, int ctas,
                           cudaStream_t st);
 cudaError_t update_occupancy(int model, int storage, bool walls, int threads, int minb, int* ctas_per_sm);
-cudaError_t launch_ghosts(int model, int storage, const GhostArgs& a, bool chained, cudaStream_t st);
+cudaError_t launch_c2f(int model, int storage, const C2FArgs& a, cudaStream_t st);
+cudaError_t launch_bc(int model, int storage, const BCArgs& a, cudaStream_t st);
+cudaError_t launch_links(int model, int storage, const LinkArgs& a, cudaStream_t st);
+cudaError_t launch_ghosts(int model, int storage, const GhostArgs& a, cudaStream_t st);  // one after the other
 cudaError_t launch_f2c(int model, int storage, const F2CArgs& a, cudaStream_t st);
 
 // dense <-> block staging for one slab of cell layers [z0, z0 + nz) of a level

@@ -179,7 +179,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
     };
     auto collide_store = [&](int c, T (&g)[Q]) {
       if constexpr (Q == 19) {
-        const T S_ = collide19<T>(g, tau0, T(a.cs2_18));
+        T S_;
+        if constexpr (std::is_same<T, double>::value) S_ = collide19_f64(g, tau0, T(a.cs2_18));
+        else S_ = collide19<T>(g, tau0, T(a.cs2_18));
         if (L.aux_dst) reinterpret_cast<T*>(L.aux_dst)[int64_t(w.block) * kCells + c] = S_;
       } else {
         if (a.force != nullptr && w.level == 0) {
@@ -208,6 +210,17 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
       }
       c += TPB;
     } while ((c & a.run_mask) >= TPB);
+  }
+}
+
+// collision of FP16 storage values (one cell or a pair)
+template <int Q, class T>
+__device__ __forceinline__ void collide_scaled(T* g, T tau0, T omega, T cs2_18, bool forced, T Fx, T Fy, T Fz, T& strain) {
+  if constexpr (Q == 19) {
+    strain = collide19<T, true>(g, tau0, cs2_18);
+  } else {
+    if (forced) collide27<T, true, true>(g, omega, Fx, Fy, Fz);
+    else collide27<T, false, true>(g, omega, T(0), T(0), T(0));
   }
 }
 
@@ -331,23 +344,35 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
           });
         }
       }
-      if constexpr (Q == 19) {
-        const V2 S_ = collide19<V2, true>(g, tau0, V2(float(a.cs2_18), float(a.cs2_18)));
-        if (L.aux_dst) {
-          float* ad = reinterpret_cast<float*>(L.aux_dst) + int64_t(w.block) * kCells + c0;
-          if (a0) ad[0] = S_.x;
-          if (a1) ad[1] = S_.y;
-        }
+      // body force of the pair (level 0 of a forced D3Q27 grid)
+      const bool forced = Q == 27 && a.force != nullptr && w.level == 0;
+      V2 F[3] = {V2(0.0), V2(0.0), V2(0.0)};
+      if (forced) {
+        const int64_t n = int64_t(L.BX) * L.BY * L.BZ * kCells;
+        const float* f = reinterpret_cast<const float*>(a.force) + int64_t(w.block) * kCells + c0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) F[k] = V2(f[k * n], f[k * n + 1]);
+      }
+      V2 strain;
+      if constexpr (W) {
+        // walled grids collide the two cells one after the other in scalar
+        // code (the compiler's contractions, so the bits of those runs, are
+        // those of a cell per thread)
+        float h0[Q], h1[Q];
+        static_for<Q>([&](auto i) {
+          h0[i] = g[i].x;
+          h1[i] = g[i].y;
+        });
+        collide_scaled<Q>(h0, tau0.x, omega.x, float(a.cs2_18), forced, F[0].x, F[1].x, F[2].x, strain.x);
+        collide_scaled<Q>(h1, tau0.x, omega.x, float(a.cs2_18), forced, F[0].y, F[1].y, F[2].y, strain.y);
+        static_for<Q>([&](auto i) { g[i] = V2(h0[i], h1[i]); });
       } else {
-        if (a.force != nullptr && w.level == 0) {
-          const int64_t n = int64_t(L.BX) * L.BY * L.BZ * kCells;
-          const int64_t j = int64_t(w.block) * kCells + c0;
-          const float* F = reinterpret_cast<const float*>(a.force);
-          collide27<V2, true, true>(g, omega, V2(F[j], F[j + 1]), V2(F[n + j], F[n + j + 1]),
-                                    V2(F[2 * n + j], F[2 * n + j + 1]));
-        } else {
-          collide27<V2, false, true>(g, omega, V2(0.0), V2(0.0), V2(0.0));
-        }
+        collide_scaled<Q>(g, tau0, omega, V2(float(a.cs2_18), float(a.cs2_18)), forced, F[0], F[1], F[2], strain);
+      }
+      if (Q == 19 && L.aux_dst) {
+        float* ad = reinterpret_cast<float*>(L.aux_dst) + int64_t(w.block) * kCells + c0;
+        if (a0) ad[0] = strain.x;
+        if (a1) ad[1] = strain.y;
       }
       S* q = dst + c0;
       if (a0 && a1) {
@@ -402,7 +427,7 @@ cudaError_t resident_ctas(K kernel, int tpb, int& occ, int* resident) {
 // shape's
 template <class M>
 constexpr int pair_ctas(int listed) {
-  return M::Q == 19 ? listed : listed == 8 ? 6 : listed == 7 ? 5 : 3;
+  return M::Q == 19 ? listed : listed == 8 ? 4 : listed == 7 ? 5 : 2;
 }
 template <class M, bool W, int TPB, int MINB>
 cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
