@@ -234,7 +234,7 @@ __device__ __forceinline__ void collide_scaled(T* g, T tau0, T omega, T cs2_18, 
 // masked out) store only the active cell.  Storage holds (f_i - w_i) / w_i,
 // which the collision takes and returns.  W = true: walls as in k_update; both
 // cells of a pair share their y and z faces, an x face has one of them.
-// 192 x 80 x 112 D3Q19 with walls: 27.7 us per step (a cell per thread: 33.2).
+// 192 x 80 x 112 D3Q19 with walls: 29.1 us per step (a cell per thread: 33.2).
 template <class M, int TPB, int MINB, bool W>
 __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
   using S = __half;
@@ -394,8 +394,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
 // number of resident CTAs per SM that caps the registers (higher occupancy).
 // FP16 storage runs the cell-pair kernel, whose bytes in flight come from its
 // residency: D3Q19 takes the listed caps as they are (256^3, 8 CTAs of 64
-// registers: 193 us per step, 7: 198, 6: 203, 5: 217), D3Q27 keeps 6, 5 or 3
-// (6 CTAs of 78 registers: 286 us; 7: 289, and with walls it spills).
+// registers: 193 us per step, 7: 198, 6: 203, 5: 217); D3Q27, whose packed
+// collision holds 126 registers, takes 4, 5 or 2 CTAs.
 
 // Splitting the blocks of short work lists: a launch with fewer blocks than
 // the part holds CTAs leaves SMs idle (64 blocks of a 32^3 grid on 152 SMs)
@@ -439,8 +439,8 @@ cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   a.run_mask = ((kCells / 2) >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
   // prefetch distance: three eighths of the CTAs resident at once (one CTA per
-  // block: 256^3 D3Q27 285.7 us per step, a half 288, a quarter 285, none
-  // 307, all 319; D3Q19 202.9, 202.6, 205.6, 229, 204 at 6 CTAs) or the grid
+  // block: 256^3 D3Q19 at 6 CTAs 202.9 us per step, a half 202.6, a quarter
+  // 205.6, none 229, all 204) or the grid
   // (persistent CTAs take items grid apart); a list short enough to be split
   // is resident as a whole
   a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : resident * 3 / 8;
