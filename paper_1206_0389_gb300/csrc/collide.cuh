@@ -201,7 +201,7 @@ __device__ __forceinline__ T collide19(T* g, T tau0, T cs2_18) {
 // The same collision in float64, whose pipes bound the update: the sums of the
 // two pairs of each plane serve all moments (48 additions instead of 63), the
 // squares of u serve every link, and one reciprocal of tau_total serves k and
-// |S|.  32^3 D3Q19 FP64 16.8 -> 14.3 us per step.
+// |S|.  32^3 D3Q19 FP64 16.8 -> 14.1 us per step.
 __device__ __forceinline__ double collide19_f64(double* g, double tau0, double cs2_18) {
   double s[9], d[9];
 #pragma unroll
