@@ -704,7 +704,10 @@ cudaPointerAttributes place_of(const void* p) {
   return at;
 }
 bool on_device(const void* p) { return place_of(p).type == cudaMemoryTypeDevice; }
+// (a kernel's 8-byte access to an array at an odd address, which NumPy's buffer
+// views can have, is an error; copies by the staging path take any address)
 bool in_reach(const lbm_ctx* ctx, const void* p, size_t bytes, bool write) {
+  if (uintptr_t(p) % sizeof(double) != 0) return false;
   const cudaPointerAttributes at = place_of(p);
   if (at.type == cudaMemoryTypeDevice) return at.device == ctx->device;
   return at.type == cudaMemoryTypeUnregistered && ctx->host_direct && bring_in(p, bytes, write);
@@ -725,7 +728,7 @@ int check_arrays(lbm_ctx* ctx, const double* const* p, const size_t* n, int narr
       any = true;
       CK(launch_check(p[k], (long long)n[k], 4 * k, ctx->d_flag, ctx->stream));
     } else if (device) {
-      return fail(ctx, LBM_ERR_ARG, "an array lies on another device than the context");
+      return fail(ctx, LBM_ERR_ARG, "a device array lies on another device than the context or at an odd address");
     } else if (p[k]) {
       for (size_t i = 0; i < n[k]; ++i) {
         const double v = p[k][i];

@@ -20,6 +20,10 @@ def ordinary(n, start):
     return np.empty(n + start)[start:]
 
 
+def ordinary_at_start(n, dtype=np.float64):
+    return np.empty(n, dtype=dtype)
+
+
 def registered(n, start):
     return torch.empty(n + start, dtype=torch.float64).pin_memory().numpy()[start:]
 
@@ -70,6 +74,46 @@ def test_in_place_transfers_equal_copies(nb, model, storage):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b, equal_nan=a.dtype.kind == "f")
+
+
+@pytest.mark.parametrize("nb", [(1, 1, 1), (5, 4, 3)])      # checked on the host; long enough for the device
+@pytest.mark.parametrize("offset", [1, 4])
+def test_arrays_at_odd_addresses(nb, offset):
+    """Buffer views that start off an 8-byte boundary take the copies."""
+    lbm = gpu()
+    lib = lbm.load()
+    n = 512 * nb[0] * nb[1] * nb[2]
+
+    def odd(size, dtype=np.float64):
+        a = np.frombuffer(bytearray(8 * size + offset), dtype=dtype, offset=offset)
+        assert a.ctypes.data % 8 == offset
+        return a
+
+    got = []
+    for make in (ordinary_at_start, odd):
+        rng = np.random.default_rng(7)
+        ctx = lbm.lbm_create("d3q27", "f32", nb, True, [], 1.7, 0.0)
+        rho, u, F = make(n), make(3 * n), make(3 * n)
+        rho[:] = 1.0 + 0.02 * rng.standard_normal(n)
+        u[:] = 0.05 * rng.standard_normal(3 * n)
+        F[:] = 1e-5 * rng.standard_normal(3 * n)
+        lbm._check(ctx, lib.lbm_init_equilibrium(ctx.h, 0, ptr(rho), ptr(u)))
+        lbm._check(ctx, lib.lbm_set_force(ctx.h, ptr(F)))
+        lbm.lbm_step(ctx, 2)
+        f, r, v = make(27 * n), make(n), make(3 * n)
+        lbm._check(ctx, lib.lbm_get_state(ctx.h, 0, ptr(f), f.size))
+        lbm._check(ctx, lib.lbm_set_state(ctx.h, 0, ptr(f), f.size))
+        lbm._check(ctx, lib.lbm_macroscopic(ctx.h, 0, ptr(r), ptr(v)))
+        cells, c = make(n, np.int64), make(27 * n)
+        cells[:] = rng.permutation(n)
+        lbm._check(ctx, lib.lbm_get_cells(ctx.h, 0, n, cells.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), ptr(c)))
+        lbm.lbm_adjoint_forward(ctx, 2, 0)
+        g = make(3 * n)
+        lbm._check(ctx, lib.lbm_adjoint_backward(ctx.h, ptr(f), ptr(g)))
+        got.append([a.copy() for a in (f, r, v, c, g)])
+        lbm.lbm_destroy(ctx)
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("make", [ordinary, registered])
