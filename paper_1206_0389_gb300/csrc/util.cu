@@ -140,12 +140,13 @@ __device__ __forceinline__ void moments64(const S* f, double& r, double& jx, dou
 }
 
 // a / b for three numerators: one reciprocal, each quotient corrected by its
-// residual
+// residual.  Where that is not finite (b zero or infinite, a infinite, an
+// overflow on the way) the quotient is taken by itself.
 __device__ __forceinline__ void divide3(double b, double& x, double& y, double& z) {
   const double r = 1.0 / b;
   auto q = [&](double a) {
-    const double v = a * r;
-    return fma(fma(-v, b, a), r, v);
+    const double v = a * r, c = fma(fma(-v, b, a), r, v);
+    return (__double2hiint(c) & 0x7ff00000) != 0x7ff00000 ? c : a / b;
   };
   x = q(x);
   y = q(y);

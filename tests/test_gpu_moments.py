@@ -73,3 +73,30 @@ def test_moments_of_single_cells_are_float64_sums(model, storage):
     keep[7:9] = False
     assert np.array_equal(r2[keep], rho[keep])
     lbm.lbm_destroy(ctx)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f64"])
+def test_velocity_of_diverged_cells_is_the_quotient(storage):
+    """u = j / rho of cells whose density or momentum is infinite or whose density is zero."""
+    lbm = gpu()
+    e = velocities(27).numpy()
+    px, mx = (int(np.flatnonzero((e == v).all(1))[0]) for v in ([1, 0, 0], [-1, 0, 0]))
+    raw = np.zeros((512, 27), dtype={"f32": np.float32, "f64": np.float64}[storage])
+    raw[:, px], raw[:, mx] = 0.5, -0.5              # j = (1, 0, 0)
+    raw[0, 0], raw[1, 0] = np.inf, -np.inf          # rho infinite
+    raw[2, 0] = -1.0                                # rho = 0
+    raw[3, px] = np.inf                             # rho and j_x infinite
+    ctx = lbm.lbm_create("d3q27", storage, (1, 1, 1), True, [], 1.7, 0.0)
+    lbm.lbm_set_raw_state(ctx, 0, np.ascontiguousarray(raw.T).reshape(-1).view(np.uint8))
+    lbm.lbm_stats_reset(ctx)
+    lbm.lbm_stats_accumulate(ctx)
+    g = raw.astype(np.float64)
+    with np.errstate(all="ignore"):
+        rho = 1.0 + g.sum(1)
+        want = np.stack([g[:, e[:, a] > 0].sum(1) - g[:, e[:, a] < 0].sum(1) for a in range(3)]) / rho
+    got_rho, got = lbm.lbm_macroscopic(ctx, 0)
+    mean, _, _ = lbm.lbm_stats_get(ctx, 0)
+    assert np.array_equal(got_rho.reshape(-1), rho)
+    assert np.array_equal(got.reshape(3, -1), want, equal_nan=True)
+    assert np.array_equal(mean[1:].reshape(3, -1), want, equal_nan=True)
+    lbm.lbm_destroy(ctx)
