@@ -216,10 +216,13 @@ __global__ void __launch_bounds__(kAdjTPB, sizeof(T) == 4 ? 5 : 2) k_adjoint(con
   begin_chained();
   constexpr int Q = 27;
   constexpr int QS = Q * kCells;
-  const T* __restrict__ fsrc = reinterpret_cast<const T*>(a.f_t);
-  const T* __restrict__ lin = reinterpret_cast<const T*>(a.lam_in);
-  T* __restrict__ lout = reinterpret_cast<T*>(a.lam_out);
-  T* __restrict__ gF = reinterpret_cast<T*>(a.dLdF);
+  // (no __restrict__: lambda, f_t and dL/dF are written by kernels that may
+  // still run when this one comes up, so none of them may be read as data
+  // that stays unchanged; chained.cuh)
+  const T* fsrc = reinterpret_cast<const T*>(a.f_t);
+  const T* lin = reinterpret_cast<const T*>(a.lam_in);
+  T* lout = reinterpret_cast<T*>(a.lam_out);
+  T* gF = reinterpret_cast<T*>(a.dLdF);
   const int64_t ncell = int64_t(a.BX) * a.BY * a.BZ * kCells;
   const int b = int(blockIdx.x) / kAdjCtas;
   const int c = int(blockIdx.x) % kAdjCtas * kAdjTPB + int(threadIdx.x);
@@ -263,10 +266,13 @@ __global__ void __launch_bounds__(kAdjTPB, sizeof(T) == 4 ? 5 : 2) k_adjoint(con
   }
   T Fbx = T(0), Fby = T(0), Fbz = T(0);
   collide27_adjoint<T>(g, lam, T(1) - T(a.omega), Fx, Fy, Fz, Fbx, Fby, Fbz);
+  Fbx += gF[j];
+  Fby += gF[ncell + j];
+  Fbz += gF[2 * ncell + j];
   static_for<Q>([&](auto i) { lout[pull(i)] = lam[i]; });
-  gF[j] += Fbx;
-  gF[ncell + j] += Fby;
-  gF[2 * ncell + j] += Fbz;
+  gF[j] = Fbx;
+  gF[ncell + j] = Fby;
+  gF[2 * ncell + j] = Fbz;
 }
 
 cudaError_t launch_adjoint(int storage, const AdjointArgs& a, cudaStream_t st) {

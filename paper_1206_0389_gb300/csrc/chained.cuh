@@ -1,5 +1,15 @@
 // Programmatic dependent launches: a chained launch is set up, down to resident
 // CTAs, while the kernel before it in the stream drains.
+//
+// What a chained kernel may read, and how: the launch is signalled before the
+// wait, so on a small grid the kernel after next can be resident while this
+// one still reads the buffer that the next one writes.  The wait returns when
+// the kernel before has ended and its writes are visible, to coherent loads.
+// Data that any kernel in the stream writes (states, lambda, dL/dF) is
+// therefore read after the wait, by ordinary loads alone: no ld.global.nc,
+// no __ldg and no __restrict__ from which the compiler may make one, all of
+// which promise data unchanged for the kernel's whole life.  Work items and
+// masks are written once, before the first launch, and may be read either way.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -37,19 +37,22 @@
 
 namespace lbm {
 
-// read-only half load that asks L2 to fetch the surrounding 256 bytes
-__device__ __forceinline__ __half ldg_half_l2(const __half* p) {
+// Loads of the state that ask L2 to fetch the surrounding 256 bytes (the pulls
+// of a warp's next rows then find their sectors in L2: 0.5225 -> 0.5203 ms per
+// 256^3 D3Q27 FP32 step).  Ordinary coherent loads, kept after the wait of a
+// chained launch: the kernel before writes this state while this one is
+// already resident (chained.cuh).
+__device__ __forceinline__ __half load_state(const __half* p) {
   unsigned short v;
-  asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
+  asm volatile("ld.global.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
   return __ushort_as_half(v);
 }
-// the same for float storage (the pulls of a warp's next rows then find
-// their sectors in L2: 0.5225 -> 0.5203 ms per 256^3 D3Q27 FP32 step)
-__device__ __forceinline__ float ldg_f32_l2(const float* p) {
+__device__ __forceinline__ float load_state(const float* p) {
   float v;
-  asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ double load_state(const double* p) { return *p; }
 
 // Start of an update kernel (chained.cuh).  With the graphs of 16 steps: 96^3
 // D3Q27 FP32 36.9 -> 31.3 us per step, 256^3 520 -> 515 us.
@@ -96,8 +99,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
                        ? (a.walls & (((w.edges >> 2) & 15) | ((w.edges & 128) ? 16 : 0) | ((w.edges & 64) ? 32 : 0)))
                        : 0;
     const T tau0 = T(L.tau0);
-    const S* __restrict__ src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
-    S* __restrict__ dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
+    const S* src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
+    S* dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
     // source of population i for cell c: base(e_z) + c + i*512 - (e_x + 8 e_y
     // + 64 e_z) + the x / y block offsets of the faces the pull crosses, with
     // base(0) = src, base(+1) = the block below for z == 0 (else src),
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
             else if (cy && cz) q = p + (iyz * kCells - ex + X);
             else if (cy) q = (ez == 1 ? b1 : ez == -1 ? bm : p) + (iy * kCells - (ex + 64 * ez) + X);
             else q = p + (iz * kCells - (ex + 8 * ey) + X + Y);
-            g[i] = St::template get<Q, i>(q);
+            g[i] = *q;
           }
         }
       });
@@ -201,10 +204,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update(const UpdateArgs a) {
     do {
       if (active(c)) {
         T g[Q];
-        pull(c, [&](auto i, const S* p) {
-          if constexpr (std::is_same<S, float>::value) g[i] = ldg_f32_l2(p);
-          else g[i] = St::template get<Q, i>(p);
-        });
+        pull(c, [&](auto i, const S* p) { g[i] = load_state(p); });
         if constexpr (W) if (wf) wall_fix(c, g);
         collide_store(c, g);
       }
@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
                        ? (a.walls & (((w.edges >> 2) & 15) | ((w.edges & 128) ? 16 : 0) | ((w.edges & 64) ? 32 : 0)))
                        : 0;  // as in k_update
     const V2 tau0 = V2(float(L.tau0), float(L.tau0)), omega = V2(float(L.omega), float(L.omega));
-    const S* __restrict__ src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
-    S* __restrict__ dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
+    const S* src = reinterpret_cast<const S*>(L.src) + int64_t(w.block) * QS;
+    S* dst = reinterpret_cast<S*>(L.dst) + int64_t(w.block) * QS;
     auto active = [&](int c) {
       if (w.mask < 0) return true;
       const uint32_t m = __ldg(a.masks + w.mask * 16 + (c >> 5));
@@ -300,12 +300,12 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
         const S* b = ez == 1 ? b1 : ez == -1 ? bm : p0;
         if constexpr (ex == 0) {
           // both sources adjacent at an even element offset: one half2 load
-          const __half2 h = __ldg(reinterpret_cast<const __half2*>(b + o + k));
+          const __half2 h = *reinterpret_cast<const __half2*>(b + o + k);
           g[i] = V2(__low2float(h), __high2float(h));
         } else if constexpr (ex == 1) {
-          g[i] = V2(__half2float(ldg_half_l2(b + o + k + Xm0)), __half2float(ldg_half_l2(b + o + k + 1)));
+          g[i] = V2(__half2float(load_state(b + o + k + Xm0)), __half2float(load_state(b + o + k + 1)));
         } else {
-          g[i] = V2(__half2float(ldg_half_l2(b + o + k)), __half2float(ldg_half_l2(b + o + k + 1 + Xp1)));
+          g[i] = V2(__half2float(load_state(b + o + k)), __half2float(load_state(b + o + k + 1 + Xp1)));
         }
       });
       if constexpr (W) {
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
                 constexpr int iy = Lattice<Q>::index(ex, -ey, ez);
                 constexpr int iz = Lattice<Q>::index(ex, ey, -ez);
                 constexpr int iyz = Lattice<Q>::index(ex, -ey, -ez);
-                const __half2 back = __ldg(reinterpret_cast<const __half2*>(p0 + ib * kCells));
+                const __half2 back = *reinterpret_cast<const __half2*>(p0 + ib * kCells);
                 V2 v = g[i];
                 if ((cy && !sy) || (cz && !sz)) {
                   v = V2(__low2float(back), __high2float(back));
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
                   if (cy && cz) q = p0 + (iyz * kCells - ex);
                   else if (cy) q = (ez == 1 ? b1 : ez == -1 ? bm : p0) + (iy * kCells - (ex + 64 * ez));
                   else q = p0 + (iz * kCells - (ex + 8 * ey) + (ey == 1 ? Ym : ey == -1 ? Yp : 0));
-                  v = V2(__half2float(__ldg(q + (ex == 1 ? Xm0 : 0))), __half2float(__ldg(q + 1 + (ex == -1 ? Xp1 : 0))));
+                  v = V2(__half2float(q[ex == 1 ? Xm0 : 0]), __half2float(q[1 + (ex == -1 ? Xp1 : 0)]));
                 }
                 if (cx && ex == 1) v.x = __low2float(back);
                 if (cx && ex == -1) v.y = __high2float(back);
