@@ -28,6 +28,13 @@ def _in_place(t):
     return t.is_cuda and torch.cuda.device_count() == 1
 
 
+def _plain(t):
+    """t as float64 values in a row of memory.  (A tensor may carry a pending
+    sign, torch.Tensor.is_neg, that neither double() nor contiguous() resolves
+    when type and layout are right already.)"""
+    return t.detach().double().contiguous().resolve_neg()
+
+
 def _call(fn, ctx, *args):
     """A C entry point on float64 device tensors.  The library works on the
     context's stream, so the current stream's work on them (their making, or
@@ -47,7 +54,7 @@ class ForcedFclb(torch.autograd.Function):
             raise ValueError("F holds %d values, the grid needs %d" % (F.numel(), 3 * ctx.ncells(0)))
         in_place = _in_place(F)
         if in_place:
-            Fd = F.detach().double().contiguous()
+            Fd = _plain(F)
             _call("lbm_set_force", ctx, Fd)
         else:
             lbm.lbm_set_force(ctx, F.detach().cpu().double().numpy())
@@ -70,7 +77,7 @@ class ForcedFclb(torch.autograd.Function):
         ctx = fctx.lbm_ctx
         if _in_place(grad_fT):
             NX, NY, NZ = ctx.dims(0)
-            lam = grad_fT.detach().double().contiguous()
+            lam = _plain(grad_fT)
             g = torch.empty((3, NZ, NY, NX), dtype=torch.float64, device=grad_fT.device)
             _call("lbm_adjoint_backward", ctx, lam, g)
         else:
