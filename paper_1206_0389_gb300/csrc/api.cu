@@ -751,7 +751,9 @@ int cur_parity(const lbm_ctx* ctx, int level) { return level == 0 ? ctx->parity0
 // one launch where the device reaches all of the caller's arrays, else slab
 // by slab through a staging buffer.  hin[c] / hout[c] are the arrays of the
 // comps components ([NZ][NY][NX] each); a NULL input component is fill[c]
-// everywhere.
+// everywhere.  One array out of reach sends all of them through the staging
+// buffer, so an array there can be on the host or on the device: the copies
+// take their direction from the addresses.
 int slab_transfer(lbm_ctx* ctx, int level, int mode, const double* const* hin, double* const* hout,
                   int comps, const double* fill = nullptr, void* raw = nullptr, double scale = 1.0) {
   const LevelPlan& lp = ctx->plan.lv[level];
@@ -779,7 +781,7 @@ int slab_transfer(lbm_ctx* ctx, int level, int mode, const double* const* hin, d
       if (hin && hin[c]) {
         a.in[c] = direct ? hin[c] : st;
         if (!direct)
-          CK(cudaMemcpyAsync(st, hin[c] + z0 * plane, cnt * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+          CK(cudaMemcpyAsync(st, hin[c] + z0 * plane, cnt * sizeof(double), cudaMemcpyDefault, ctx->stream));
       }
       if (fill) a.fill[c] = fill[c];
       if (hout) a.out[c] = direct ? hout[c] : st;
@@ -804,8 +806,8 @@ int slab_transfer(lbm_ctx* ctx, int level, int mode, const double* const* hin, d
     CK(launch_slab(ctx->model, ctx->storage, a, ctx->stream));
     if (hout && !direct)
       for (int c = 0; c < comps; ++c)
-        CK(cudaMemcpyAsync(hout[c] + z0 * plane, ctx->stage + c * cnt, cnt * sizeof(double),
-                           cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaMemcpyAsync(hout[c] + z0 * plane, ctx->stage + c * cnt, cnt * sizeof(double), cudaMemcpyDefault,
+                           ctx->stream));
   }
   CK(cudaStreamSynchronize(ctx->stream));
   return LBM_OK;
