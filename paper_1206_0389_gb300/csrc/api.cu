@@ -99,6 +99,8 @@ struct lbm_ctx {
   // graphs of one and of kManySteps coarse steps, one per level-0 parity
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
   bool graphs_valid = false;
+  int step_ops = 0;          // launches of a coarse step
+  int64_t graph_steps = 0;   // coarse steps run by lbm_step since the graphs were last captured
   bool profiling = false;
   // adjoint: checkpoints every `every` steps, segment buffers, lambda, dL/dF
   int adj_T = 0, adj_every = 0;
@@ -457,6 +459,13 @@ int restrict_all(lbm_ctx* ctx) {
 // step, so a run of steps goes out as graphs of kManySteps steps: 53,760 cells
 // of D3Q27 FP32 8.4 -> 4.4 us per step, 96^3 36.9 -> 31.3, 256^3 FP16 309 -> 300
 // (with chained launches).  The number is even: the parity comes round.
+// A graph of that many steps is captured once the steps since the last change
+// of the inflow, outlet or force (those of the running call included) reach
+// kManySteps times the launches of a step: about what its capture costs in
+// steps saved.  Capture against gain per step, us: one periodic level (1
+// launch) 55 and 3.6, open (2) 100 and 3, three levels (11 or 14) 1100 to 1450
+// and 3.5 to 7.  A program that changes the inflow every 16 steps paid each
+// time: 16 steps of a 3-level FP32 grid 2562 -> 1680 us, FP16 2696 -> 1485.
 constexpr int kManySteps = 16;
 
 // captures `steps` coarse steps that start at level-0 parity p0
@@ -541,11 +550,13 @@ int capture_steps(lbm_ctx* ctx, int p0, int steps, cudaGraphExec_t* exec) {
   return LBM_OK;
 }
 
-// the graphs of single steps; those of kManySteps are captured when first used
+// the graphs of single steps; those of kManySteps are captured when they pay
 int build_graphs(lbm_ctx* ctx) {
   drop_graphs(ctx);
   for (int p = 0; p < 2; ++p)
     if (int rc = capture_steps(ctx, p, 1, &ctx->graph[p])) return rc;
+  ctx->step_ops = int(build_schedule(ctx, 0).size());
+  ctx->graph_steps = 0;
   ctx->graphs_valid = true;
   return LBM_OK;
 }
@@ -1158,11 +1169,12 @@ int lbm_step(lbm_ctx* ctx, int coarse_steps) {
     if (rc) return rc;
   }
   int left = coarse_steps;
-  if (left >= kManySteps && !ctx->many[ctx->parity0]) {
+  ctx->graph_steps += coarse_steps;
+  if (left >= kManySteps && !ctx->many[ctx->parity0] && ctx->graph_steps >= int64_t(kManySteps) * ctx->step_ops) {
     int rc = capture_steps(ctx, ctx->parity0, kManySteps, &ctx->many[ctx->parity0]);
     if (rc) return rc;
   }
-  for (; left >= kManySteps; left -= kManySteps) {
+  for (; left >= kManySteps && ctx->many[ctx->parity0]; left -= kManySteps) {
     CK(cudaGraphLaunch(ctx->many[ctx->parity0], ctx->stream));
     ctx->step += kManySteps;
   }
