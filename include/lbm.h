@@ -316,10 +316,11 @@ int lbm_adjoint_backward(lbm_ctx* ctx, const double* dLdf_T, double* dLdF);
 
 /* Kernel timing: when enabled, lbm_step launches kernels directly (no graph)
  * between CUDA events on the context stream and accumulates per-kind device
- * time.  kinds: 0 update (stream-collide), 1 coarse-to-fine (with the boundary
- * ghosts and nozzle links of the same substep), 2 fine-to-coarse, 3 boundary, 4 other (nothing of a step; an lbm_adjoint_backward call adds the device time of
- * its recompute + adjoint sweep here as one entry).  ms[k] total
- * milliseconds, launches[k] launch counts. */
+ * time.  kinds: 0 update (stream-collide), 1 coarse-to-fine, 2 fine-to-coarse,
+ * 3 boundary (inflow and outlet ghosts, nozzle links), 4 other (nothing of a
+ * step; an lbm_adjoint_backward call adds the device time of its recompute +
+ * adjoint sweep here as one entry).  ms[k] total milliseconds, launches[k]
+ * launch counts. */
 int lbm_set_profiling(lbm_ctx* ctx, int enable);
 int lbm_get_profile(lbm_ctx* ctx, double ms[5], int64_t launches[5]);
 

@@ -22,6 +22,7 @@
 #include <cstring>
 #include <string>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "kernels.cuh"
@@ -421,14 +422,26 @@ cudaError_t run_op(lbm_ctx* c, const Op& op, cudaStream_t st, bool chained = fal
   return cudaErrorInvalidValue;
 }
 
-// kinds of lbm_get_profile (ghosts of several kinds count as coarse-to-fine)
-int op_kind_index(const Op& op) {
-  switch (op.kind) {
-    case Op::GHOSTS: return op.ga.c2f.n > 0 ? 1 : 3;
-    case Op::UPDATE: return 0;
-    case Op::F2C: return 2;
+// the launches of an op one by one, each with its kind in lbm_get_profile
+std::vector<std::pair<int, Op>> op_launches(const Op& op) {
+  if (op.kind == Op::F2C) return {{2, op}};
+  if (op.kind == Op::UPDATE && op.ua.nitems > 0) return {{0, op}};
+  std::vector<std::pair<int, Op>> out;
+  Op one = op;
+  one.ga = GhostArgs{};
+  if (op.ga.c2f.n > 0) {
+    out.emplace_back(1, one);
+    out.back().second.ga.c2f = op.ga.c2f;
   }
-  return 4;
+  if (op.ga.bc.n > 0) {
+    out.emplace_back(3, one);
+    out.back().second.ga.bc = op.ga.bc;
+  }
+  if (op.ga.link.n > 0) {
+    out.emplace_back(3, one);
+    out.back().second.ga.link = op.ga.link;
+  }
+  return out;
 }
 
 // restriction of every hidden layer from the current fine state (after an
@@ -1146,17 +1159,17 @@ int lbm_step(lbm_ctx* ctx, int coarse_steps) {
     CK(cudaEventCreate(&e1));
     for (int n = 0; n < coarse_steps; ++n) {
       std::vector<Op> ops = build_schedule(ctx, ctx->parity0);
-      for (const Op& op : ops) {
-        CK(cudaEventRecord(e0, ctx->stream));
-        CK(run_op(ctx, op, ctx->stream));
-        CK(cudaEventRecord(e1, ctx->stream));
-        CK(cudaEventSynchronize(e1));
-        float ms = 0;
-        CK(cudaEventElapsedTime(&ms, e0, e1));
-        const int k = op_kind_index(op);
-        ctx->prof_ms[k] += ms;
-        ctx->prof_n[k] += 1;
-      }
+      for (const Op& op : ops)
+        for (const auto& [kind, launch] : op_launches(op)) {
+          CK(cudaEventRecord(e0, ctx->stream));
+          CK(run_op(ctx, launch, ctx->stream));
+          CK(cudaEventRecord(e1, ctx->stream));
+          CK(cudaEventSynchronize(e1));
+          float ms = 0;
+          CK(cudaEventElapsedTime(&ms, e0, e1));
+          ctx->prof_ms[kind] += ms;
+          ctx->prof_n[kind] += 1;
+        }
       ctx->parity0 ^= 1;
       ctx->step++;
     }
