@@ -97,6 +97,7 @@ struct lbm_ctx {
   uint64_t seed = 0;
   // launch configuration
   int threads = 256, minb = 1, ctas = 0;
+  int resident = 0;  // CTAs of that shape that the part holds at once
   // graphs of one and of kManySteps coarse steps, one per level-0 parity
   cudaGraphExec_t graph[2] = {nullptr, nullptr}, many[2] = {nullptr, nullptr};
   bool graphs_valid = false;
@@ -349,6 +350,7 @@ std::vector<Op> build_schedule(lbm_ctx* c, int p0) {
     u.slip = c->plan.slip;
     // only the inflow reads the step counter, before the last update
     u.step_inc = k == K - 1 && !c->plan.periodic_x ? c->d_step : nullptr;
+    u.resident = c->resident;
     up.k = k;
     if (branch0) {
       // the first substep updates level 0 in launches of its own: the fine
@@ -618,7 +620,8 @@ int autotune(lbm_ctx* ctx) {
     const int t = sh[0], mb = sh[1];
     int occ = 0;
     if (update_occupancy(ctx->model, ctx->storage, ctx->plan.walls != 0, t, mb, &occ) != cudaSuccess || occ < 1) continue;
-    const int clist[2] = {0, occ * ctx->sms};
+    trial.resident = occ * ctx->sms;
+    const int clist[2] = {0, trial.resident};
     for (int cc : clist) {
       // a list that is resident as a whole makes the same launch either way
       if (cc > 0 && trial.nitems <= (ctx->storage == LBM_F64 ? cc / 4 : cc)) continue;
@@ -1034,6 +1037,10 @@ int create_context(lbm_ctx** out, lbm_model model, lbm_storage storage, const lb
   ce = cudaStreamSynchronize(ctx->stream);
   if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("init: ") + cudaGetErrorString(ce));
   if (int rc = autotune(ctx); rc != LBM_OK) return bail(rc, "autotune: " + ctx->err);
+  int per_sm = 0;
+  ce = update_occupancy(ctx->model, ctx->storage, ctx->plan.walls != 0, ctx->threads, ctx->minb, &per_sm);
+  if (ce != cudaSuccess) return bail(LBM_ERR_CUDA, std::string("occupancy: ") + cudaGetErrorString(ce));
+  ctx->resident = per_sm * ctx->sms;
   // the tuning runs wrote the second buffers; clear them again
   for (int l = 0; l < ctx->L; ++l) {
     const size_t fb = size_t(ctx->plan.lv[l].nblocks()) * 512 * ctx->Q * sb;

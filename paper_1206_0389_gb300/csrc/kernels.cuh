@@ -60,8 +60,8 @@ struct UpdateArgs {
                           // the faces x = 0 / x = NX, no-slip) and the free-slip ones
                           // among the y/z walls; read by the W = true kernels
   int pf_ahead;           // FP16 kernels: a CTA asks L2 for the block of work item
-                          // it + pf_ahead (about half a wave ahead); 0 = off (set by
-                          // the launcher)
+                          // it + pf_ahead (set by the launcher; 0 = off)
+  int resident;           // CTAs of the launch shape that the part holds at once
   int split;              // log2 of the runs a block's cells are cut into, each the work
                           // of one CTA (set by the launcher)
   long long* step_inc;    // coarse-step counter that the last update of a coarse step

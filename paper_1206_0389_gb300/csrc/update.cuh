@@ -412,17 +412,6 @@ inline int split_for(int nitems, int max_runs, int resident, bool always) {
   return s;
 }
 
-template <class K>
-cudaError_t resident_ctas(K kernel, int tpb, int& occ, int* resident) {
-  cudaError_t e = cudaSuccess;
-  if (occ == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, tpb, 0);
-  int dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  *resident = occ * sms;
-  return e;
-}
-
 // CTAs per SM that the cell-pair kernel is compiled for in place of a listed
 // shape's
 template <class M>
@@ -431,11 +420,7 @@ constexpr int pair_ctas(int listed) {
 }
 template <class M, bool W, int TPB, int MINB>
 cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
-  static int occ = 0;  // CTAs per SM of this instance (a property of the kernel)
-  int resident = 0;
-  cudaError_t e = resident_ctas(k_update_pair<M, TPB, MINB, W>, TPB, occ, &resident);
-  if (e != cudaSuccess) return e;
-  a.split = split_for(a.nitems, kCells / 2 / TPB, resident, false);
+  a.split = split_for(a.nitems, kCells / 2 / TPB, a.resident, false);
   a.run_mask = ((kCells / 2) >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
   // prefetch distance: three eighths of the CTAs resident at once (one CTA per
@@ -443,7 +428,7 @@ cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   // 205.6, none 229, all 204) or the grid
   // (persistent CTAs take items grid apart); a list short enough to be split
   // is resident as a whole
-  a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : resident * 3 / 8;
+  a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : a.resident * 3 / 8;
   return launch_chained(k_update_pair<M, TPB, MINB, W>, grid, TPB, a, a.chained, st);
 }
 template <class M, bool W>
@@ -467,11 +452,7 @@ cudaError_t occ_pair(int threads, int minb, int* n) {
 
 template <class M, class S, bool W, int TPB, int MINB>
 cudaError_t launch_shape(UpdateArgs a, int ctas, cudaStream_t st) {
-  static int occ = 0;
-  int resident = 0;
-  cudaError_t e = resident_ctas(k_update<M, S, TPB, MINB, W>, TPB, occ, &resident);
-  if (e != cudaSuccess) return e;
-  a.split = split_for(a.nitems, kCells / TPB, resident, std::is_same<S, double>::value);
+  a.split = split_for(a.nitems, kCells / TPB, a.resident, std::is_same<S, double>::value);
   a.run_mask = (kCells >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
   return launch_chained(k_update<M, S, TPB, MINB, W>, grid, TPB, a, a.chained, st);
