@@ -48,10 +48,10 @@ def _call(fn, ctx, *args):
 class ForcedFclb(torch.autograd.Function):
     @staticmethod
     def forward(fctx, F, ctx, f0, T, every):
-        lbm.lbm_set_state(ctx, 0, np.asarray(f0, dtype=np.float64))
         NX, NY, NZ = ctx.dims(0)
         if F.numel() < 3 * ctx.ncells(0):
             raise ValueError("F holds %d values, the grid needs %d" % (F.numel(), 3 * ctx.ncells(0)))
+        lbm.lbm_set_state(ctx, 0, np.asarray(f0, dtype=np.float64))
         in_place = _in_place(F)
         if in_place:
             Fd = _plain(F)

@@ -69,3 +69,10 @@ def test_force_and_gradient_reach_the_library_by_value(form, calls):
     by_name = dict(calls)
     assert np.array_equal(by_name["lbm_set_force"][0], x.reshape(-1).numpy())
     assert np.array_equal(by_name["lbm_adjoint_backward"][0], lam.reshape(-1).numpy())
+
+
+def test_short_force_is_refused_before_the_context_changes(calls):
+    F = torch.zeros(3, N, N, N - 1, dtype=torch.float64, requires_grad=True)
+    with pytest.raises(ValueError):
+        autograd.forced_fclb(F, FakeContext(), np.zeros((27, N, N, N)), 2, 1)
+    assert calls == []
