@@ -202,14 +202,16 @@ __device__ __forceinline__ void collide27_adjoint(const T* g, T* lam, T om1, T F
 
 // One adjoint step over all blocks of a periodic single level, a cell per
 // thread and four CTAs per block.  An FP32 step reads f_t, lambda and the force
-// and writes lambda and dL/dF, 360 bytes a cell, and is bound by the latency
-// of its 54 scattered loads per thread: the reverse of the lines (half the
-// instructions of a pass-by-pass reverse) fits 96 registers, 20 warps per SM
-// instead of 16, and CTAs of one cell per thread chain and even out better than
-// four cells in a row.  us per step, pass by pass -> lines -> also chained, 5
-// CTAs per SM, a cell per thread: 96^3 FP32 76.4 -> 64.1 -> 58.3 (0.80 of the
-// copy peak), 128^3 165 -> 140 -> 131, 32^3 12.4 -> 11.3 -> 5.3.  FP64 is bound by
-// the float64 pipes: 64^3 639 -> 420 -> 369.
+// and writes lambda and dL/dF, 360 bytes a cell, and is bound by HBM on large
+// grids, by the latency of its 54 scattered loads per thread on small ones: the
+// reverse of the lines (half the instructions of a pass-by-pass reverse) fits 96
+// registers, 20 warps per SM instead of 16, and CTAs of one cell per thread
+// chain and even out better than four cells in a row.  us per step, pass by
+// pass -> lines -> also chained, 5 CTAs per SM, a cell per thread -> loads of
+// dL/dF before the stores of lambda: 96^3 FP32 76.4 -> 64.1 -> 58.3 -> 50.9
+// (0.92 of the copy peak), 128^3 165 -> 140 -> 131 -> 114 (0.97), 32^3 12.4 ->
+// 11.3 -> 5.3 -> 5.3.  FP64 is bound by the float64 pipes: 64^3 639 -> 420 -> 369
+// -> 367.
 constexpr int kAdjTPB = 128, kAdjCtas = kCells / kAdjTPB;
 template <class T>
 __global__ void __launch_bounds__(kAdjTPB, sizeof(T) == 4 ? 5 : 2) k_adjoint(const AdjointArgs a) {

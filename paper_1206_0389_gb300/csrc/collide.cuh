@@ -463,20 +463,20 @@ __device__ __forceinline__ void collide27_lines(T* g, T om1, T Fx, T Fy, T Fz) {
       const T lo = g[D3Q27::index(a - 1, b - 1, -1)], hi = g[D3Q27::index(a - 1, b - 1, 1)];
       sz[a][b] = hi + lo;
       dz[a][b] = hi - lo;
-      m0[a][b] = (sz[a][b]) + g[D3Q27::index(a - 1, b - 1, 0)];
+      m0[a][b] = sz[a][b] + g[D3Q27::index(a - 1, b - 1, 0)];
     }
   T M0[3], My[3], Myy[3], Dz[3], Dyz[3], Szz[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     Myy[a] = m0[a][2] + m0[a][0];
     My[a] = m0[a][2] - m0[a][0];
-    M0[a] = (Myy[a]) + m0[a][1];
+    M0[a] = Myy[a] + m0[a][1];
     Dz[a] = (dz[a][2] + dz[a][0]) + dz[a][1];
     Dyz[a] = dz[a][2] - dz[a][0];
     Szz[a] = (sz[a][2] + sz[a][0]) + sz[a][1];
   }
   T Sxx = M0[2] + M0[0], jx = M0[2] - M0[0];
-  T drho = (Sxx) + M0[1];
+  T drho = Sxx + M0[1];
   T jy = (My[2] + My[0]) + My[1], Sxy = My[2] - My[0];
   T Syy = (Myy[2] + Myy[0]) + Myy[1];
   T jz = (Dz[2] + Dz[0]) + Dz[1], Sxz = Dz[2] - Dz[0];

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
     const LevelPtrs& L = a.lv[w.level];
     const int BX = L.BX, BXY = L.BX * L.BY;
     if (threadIdx.x == 0 && a.pf_ahead > 0 && it + a.pf_ahead < a.nitems) {
-      // the block a CTA about half a wave later takes: its whole [Q][512] run
+      // the block that a CTA pf_ahead items later takes: its whole [Q][512] run
       // (contiguous, 16-byte aligned) into L2 by one bulk prefetch of the
       // TMA unit, so that CTA's loads find L2 instead of DRAM
       const WorkItem wn = a.items[it + a.pf_ahead];
@@ -393,9 +393,9 @@ __global__ void __launch_bounds__(TPB, MINB) k_update_pair(const UpdateArgs a) {
 // Launch shapes the autotuner chooses from: threads per CTA, and a minimum
 // number of resident CTAs per SM that caps the registers (higher occupancy).
 // FP16 storage runs the cell-pair kernel, whose bytes in flight come from its
-// residency: D3Q19 takes the listed caps as they are (256^3, 8 CTAs of 64
-// registers: 193 us per step, 7: 198, 6: 203, 5: 217); D3Q27, whose packed
-// collision holds 126 registers, takes 4, 5 or 2 CTAs.
+// residency: D3Q19 takes the listed caps as they are (256^3, 8 or 7 CTAs, both
+// of 64 registers: 194 and 193 us per step, 6: 203, 5: 217); D3Q27, whose
+// packed collision holds 126 registers, takes 4, 5 or 2 CTAs.
 
 // Splitting the blocks of short work lists: a launch with fewer blocks than
 // the part holds CTAs leaves SMs idle (64 blocks of a 32^3 grid on 152 SMs)
@@ -423,11 +423,12 @@ cudaError_t launch_pair_shape(UpdateArgs a, int ctas, cudaStream_t st) {
   a.split = split_for(a.nitems, kCells / 2 / TPB, a.resident, false);
   a.run_mask = ((kCells / 2) >> a.split) - 1;
   const int units = a.nitems << a.split, grid = ctas > 0 ? std::min(ctas, units) : units;
-  // prefetch distance: three eighths of the CTAs resident at once (one CTA per
-  // block: 256^3 D3Q19 at 6 CTAs 202.9 us per step, a half 202.6, a quarter
-  // 205.6, none 229, all 204) or the grid
-  // (persistent CTAs take items grid apart); a list short enough to be split
-  // is resident as a whole
+  // prefetch distance: three eighths of the CTAs resident at once, or the grid
+  // (persistent CTAs take items grid apart); a list short enough to be split is
+  // resident as a whole.  256^3, one CTA per block, us per step at a distance
+  // of none, 1/8, 1/4, 3/8, 1/2, 3/4 and all of the residents: D3Q19 (8 CTAs
+  // per SM) 215, 202, 197, 195, 195, 203, 216; D3Q27 (4) 329, 311, 304, 300,
+  // 301, 303, 308
   a.pf_ahead = a.split > 0 ? 0 : ctas > 0 ? grid : a.resident * 3 / 8;
   return launch_chained(k_update_pair<M, TPB, MINB, W>, grid, TPB, a, a.chained, st);
 }
